@@ -22,7 +22,8 @@
 //      -> one packed 64-bit atomicMax per cell into the stage-1
 //      max-projection; statistics (SIGMA mode); the harmonic rows the
 //      harmonic sum needs are staged through shared memory and written
-//      coalesced.  In plane mode the power rows are written instead.
+//      coalesced.  In plane mode the asked-for power rows are staged the same
+//      way and written instead.
 // Each template costs two barriers over its segment's threads; the metadata
 // the epilogue and the row stores need (template index, slot-entry range and
 // entries) is prefetched one template ahead into shared memory by cp.async,
@@ -152,18 +153,21 @@ conv_kernel(ConvArgs a) {
     const SyncNamed bar_half{1 + half, NT};
     const int warp = tid >> 5;
 
-    // (spectrum, template group) entry of this CTA: binary search of the CTA prefix
-    int lo = 0, hi = a.n_work - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((int)blockIdx.x >= __ldg(&a.grp[mid].cta0)) lo = mid; else hi = mid - 1;
-    }
-    const int g = lo;
+    // (spectrum, template group) entry of this CTA
+    const int cta = (int)blockIdx.x + a.cta_base;
+    const int g = work_entry(a, cta);
     const int item = __ldg(&a.grp[g].item);
 #define itm (a.items + item)
     const int V = __ldg(&a.grp[g].V), bM = __ldg(&a.grp[g].bM);
-    const int tb = __ldg(&a.grp[g].tb), te = __ldg(&a.grp[g].te);
-    const int s = ((int)blockIdx.x - __ldg(&a.grp[g].cta0)) * SEGS + half;
+    int tb = __ldg(&a.grp[g].tb), te = __ldg(&a.grp[g].te);
+    if constexpr (MODE == 1) {
+        // plane rows: only the asked-for templates of the group are filtered
+        const int g1 = te;
+        te = first_at_least(a.order, tb, g1, a.t0 + a.nt);
+        tb = first_at_least(a.order, tb, te, a.t0);
+        if (tb >= te) return;                                 // (uniform over the CTA, nothing set up yet)
+    }
+    const int s = (cta - __ldg(&a.grp[g].cta0)) * SEGS + half;
     const int seg0 = s * V;                                   // first output cell (< 2^31: max_bins <= 2^29)
 
     if (tid < NBUF) {
@@ -360,14 +364,15 @@ conv_kernel(ConvArgs a) {
             }
             cp_async_commit();
         }
-        if constexpr (MODE == 0)
-            if (k > tb) {
-                // the previous template's staged row
-                const TplMeta mp = tq[half][(k - 1) & 3];
-                if (mp.e0 < mp.e1)
-                    store_rows(a, rent[half][(k - 1) & 1], mp.e1 - mp.e0, stage, sbound[half], (int)seg0, j, NT,
-                               kChkRowStore);
-            }
+        if (k > tb) {
+            // the previous template's staged row
+            const TplMeta mp = tq[half][(k - 1) & 3];
+            if constexpr (MODE == 1)
+                store_plane_row(a, mp.t, stage, seg0, V, itm->bN, j, NT, kChkPlaneStore);
+            else if (mp.e0 < mp.e1)
+                store_rows(a, rent[half][(k - 1) & 1], mp.e1 - mp.e0, stage, sbound[half], (int)seg0, j, NT,
+                           kChkRowStore);
+        }
         fft_rest<LOG2L, +1>(v, work, j, twi, bar_half);
         float P[16];
 #pragma unroll
@@ -430,20 +435,20 @@ conv_kernel(ConvArgs a) {
                         stage[swzf(rv + NT * r)] = P[r];
                 }
             }
-        } else if (tq[half][k & 3].t >= a.t0 && tq[half][k & 3].t < a.t0 + a.nt) {
-            const int t = tq[half][k & 3].t;
-            const int64_t row0 = (int64_t)(t - a.t0) * (2 * (int64_t)a.items[0].N) + seg0;
-            float *row = a.plane + row0;
+        } else {
 #pragma unroll
-            for (int r = 0; r < RK; ++r)
-                if (((vmask >> r) & 1u) && JERK_CHECK(row0 + rv + NT * r < a.plane_len, a.chk, kChkPlaneStore))
-                    row[rv + NT * r] = P[r];
+            for (int r = 0; r < RK; ++r) {
+                if constexpr (NT % 256 == 0)
+                    stage[swzf(rv) + NT * r] = P[r];
+                else
+                    stage[swzf(rv + NT * r)] = P[r];
+            }
         }
     }
     };
     if constexpr (LOG2L <= 12) {
         // (at L = 8192 the three copies spill)
-        const int rd = MODE == 0 ? 16 - (V + NT - 1) / NT : 0;
+        const int rd = 16 - (V + NT - 1) / NT;
         if (rd >= 2)
             template_loop(std::integral_constant<int, 2>{});
         else if (rd == 1)
@@ -455,10 +460,12 @@ conv_kernel(ConvArgs a) {
     }
 
     cp_async_wait_all();
-    if constexpr (MODE == 0) {
-        bar_half();
-        if (!failed && te > tb) {
-            const TplMeta mp = tq[half][(te - 1) & 3];
+    bar_half();
+    if (!failed && te > tb) {
+        const TplMeta mp = tq[half][(te - 1) & 3];
+        if constexpr (MODE == 1) {
+            store_plane_row(a, mp.t, stage, seg0, V, itm->bN, j, NT, kChkPlaneStore);
+        } else {
             if (mp.e0 < mp.e1)
                 store_rows(a, rent[half][(te - 1) & 1], mp.e1 - mp.e0, stage, sbound[half], (int)seg0, j, NT,
                            kChkRowStore);

@@ -208,16 +208,20 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
     const int row = 32 * quarter + lane;                      // operand / accumulator row: (seg, r)
     const int seg = row >> 6, r = row & 63;
 
-    // (spectrum, template group) entry of this CTA: binary search of the CTA prefix
-    int lo = 0, hi = a.n_work - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((int)blockIdx.x >= __ldg(&a.grp[mid].cta0)) lo = mid; else hi = mid - 1;
-    }
+    // (spectrum, template group) entry of this CTA
+    const int cta = (int)blockIdx.x + a.cta_base;
+    const int lo = work_entry(a, cta);
     const ItemDesc *itm = a.items + __ldg(&a.grp[lo].item);
     const int V = __ldg(&a.grp[lo].V), bM = __ldg(&a.grp[lo].bM);
-    const int tb = __ldg(&a.grp[lo].tb), te = __ldg(&a.grp[lo].te);
-    const int s_base = ((int)blockIdx.x - __ldg(&a.grp[lo].cta0)) * SEGS;
+    int tb = __ldg(&a.grp[lo].tb), te = __ldg(&a.grp[lo].te);
+    if constexpr (MODE == 1) {
+        // plane rows: only the asked-for templates of the group are filtered
+        const int g1 = te;
+        te = first_at_least(a.order, tb, g1, a.t0 + a.nt);
+        tb = first_at_least(a.order, tb, te, a.t0);
+        if (tb >= te) return;                                 // (uniform over the CTA, nothing set up yet)
+    }
+    const int s_base = (cta - __ldg(&a.grp[lo].cta0)) * SEGS;
     const int64_t bN = itm->bN;
 
     if (tid == 0) {
@@ -535,15 +539,13 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
                 }
             }
         } else {
-            if (t >= a.t0 && t < a.t0 + a.nt) {
-                const int64_t row0 = (int64_t)(t - a.t0) * bN + seg0;
-                float *prow = a.plane + row0;
+            const int64_t row0 = (int64_t)(t - a.t0) * bN + seg0;
+            float *prow = a.plane + row0;
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    if (i < nvalid &&
-                        JERK_CHECK(row0 + 64 * (16 * gcol + i) + r < a.plane_len, a.chk, kChkTcPlaneStore))
-                        prow[64 * (16 * gcol + i) + r] = P[i] * psc;
-            }
+            for (int i = 0; i < 16; ++i)
+                if (i < nvalid &&
+                    JERK_CHECK(row0 + 64 * (16 * gcol + i) + r < a.plane_len, a.chk, kChkTcPlaneStore))
+                    prow[64 * (16 * gcol + i) + r] = P[i] * psc;
         }
     };
 

@@ -59,6 +59,7 @@ struct ConvArgs {
     const ConvGroup *grp;    // [n_work + 1] (item, group) entries; grp[n_work].cta0 = total CTAs
     int32_t T, n_work;
     int32_t t0, nt;          // template range written in plane mode
+    int32_t cta_base;        // CTA of the work list that block 0 is (plane mode skips leading groups)
     // search mode
     const int32_t *slot_beg; // [T + 1] CSR into the slot entries
     const int32_t *slot_h;
@@ -90,6 +91,26 @@ __device__ __forceinline__ bool inject_at(const ConvArgs &a, int mode, int pos) 
 #else
 __device__ __forceinline__ bool inject_at(const ConvArgs &, int, int) { return false; }
 #endif
+
+// Work entry (spectrum, template group) of a CTA: binary search of the CTA prefix.
+__device__ __forceinline__ int work_entry(const ConvArgs &a, int cta) {
+    int lo = 0, hi = a.n_work - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (cta >= __ldg(&a.grp[mid].cta0)) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// First position k in [lo, hi) whose template index is at least t, or hi (a
+// group's positions are in ascending template order).
+__device__ __forceinline__ int first_at_least(const int32_t *order, int lo, int hi, int t) {
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(order + mid) < t) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
 
 // Sites of the debug build's bounds checks (the first failing one is recorded).
 enum CheckSite {

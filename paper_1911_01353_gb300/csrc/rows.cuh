@@ -59,4 +59,38 @@ __device__ __forceinline__ void store_rows(const ConvArgs &a, const RowEntries &
     }
 }
 
+// Plane mode: the staged power row of template t (cell c of the segment at
+// pw[swzf(c)]) to its row of the plane, cells c < V inside the spectrum.
+// Rows are 2 n floats apart and the plane is the caller's, so a row starts on
+// a 16-, 8- or 4-byte boundary: the widest store that its address allows.
+// Coalesced like this, 64 rows of a 2^18-bin spectrum are written at the rate
+// they are filtered; from the registers, whose cells are digit-reversed over
+// the lanes, each 4-byte store was a 32-byte sector of its own.
+__device__ __forceinline__ void store_plane_row(const ConvArgs &a, int t, const float *pw, int s0, int V, int64_t bN,
+                                                int j, int nt, int site) {
+    const int64_t row0 = (int64_t)(t - a.t0) * bN + s0;
+    const int64_t left = bN - s0;
+    const int n = left < V ? (int)left : V;
+    if (n <= 0) return;                                       // a CTA's last segment may lie past the spectrum
+    float *dst = a.plane + row0;
+    const unsigned align = (unsigned)(reinterpret_cast<uintptr_t>(dst) & 15u);
+    if (align == 0) {
+        for (int g = j; g < (n >> 2); g += nt)
+            if (JERK_CHECK(row0 + 4 * g + 3 < a.plane_len, a.chk, site))
+                *reinterpret_cast<float4 *>(dst + 4 * g) = row4(pw, g);
+        for (int c = (n & ~3) + j; c < n; c += nt)
+            if (JERK_CHECK(row0 + c < a.plane_len, a.chk, site)) dst[c] = pw[swzf(c)];
+    } else if (align == 8) {
+        // (a pair of cells stays together under swzf)
+        for (int g = j; g < (n >> 1); g += nt)
+            if (JERK_CHECK(row0 + 2 * g + 1 < a.plane_len, a.chk, site))
+                *reinterpret_cast<float2 *>(dst + 2 * g) = *reinterpret_cast<const float2 *>(pw + swzf(2 * g));
+        for (int c = (n & ~1) + j; c < n; c += nt)
+            if (JERK_CHECK(row0 + c < a.plane_len, a.chk, site)) dst[c] = pw[swzf(c)];
+    } else {
+        for (int c = j; c < n; c += nt)
+            if (JERK_CHECK(row0 + c < a.plane_len, a.chk, site)) dst[c] = pw[swzf(c)];
+    }
+}
+
 }  // namespace jerk
