@@ -169,10 +169,12 @@ struct PeakArgs {
 
 // launchers (return cudaGetLastError())
 cudaError_t launch_normalise(const float2 *in, float2 *out, int64_t n, int block, cudaStream_t st);
+size_t tap_table_elems(int bM);
+cudaError_t launch_tap_table(double2 *tab, const double2 *gl, int b, int bM, int pad, cudaStream_t st);
 cudaError_t launch_taps(const int32_t *zt, const int32_t *wt, const int32_t *tlist, int32_t t0, int32_t nt, int b,
-                        int pad, int bM, const double2 *gl, int n_gl, double2 *out, cudaStream_t st);
-cudaError_t launch_template_fft(const double2 *taps, const int32_t *shift, const int32_t *klen, int32_t nt, int K,
-                                int L, const double2 *tw, int fold_r0, float2 *bank, cudaStream_t st);
+                        int pad, int bM, const double2 *gl, const double2 *tab, double2 *out, cudaStream_t st);
+cudaError_t launch_template_fft(const double2 *taps, const int32_t *dest, const int32_t *offs, int32_t n, int bM,
+                                int L, const double2 *tw, int fold_r0, float2 *bank, float *cmax, cudaStream_t st);
 int conv_fold_radix(int log2L);      // radix of the FP32 filter's first inverse pass (the bank's folded form)
 // the tensor-core filter's bank pairs spectrum values f and f + kTcBankPair
 // (the two rows of a DFT block one thread multiplies together)
@@ -180,7 +182,6 @@ constexpr int kTcBankPair = 64;
 cudaError_t launch_twiddles64(double2 *tw, int L, cudaStream_t st);
 cudaError_t launch_conv(int log2L, int mode, bool stats, const ConvArgs &a, int n_ctas, cudaStream_t st);
 cudaError_t launch_conv_tc(int precision, int mode, bool stats, const ConvArgs &a, int n_ctas, cudaStream_t st);
-cudaError_t launch_bank_maxabs(const float2 *bank, int64_t n, float *out, int sms, cudaStream_t st);
 int conv_segs_per_cta(int log2L);
 cudaError_t launch_harmonic(const HarmArgs &a, int nblk_y, bool stats, cudaStream_t st);
 int harmonic_cells_per_block();
@@ -233,7 +234,7 @@ struct BankShare {
     float2 *d_bank = nullptr;
     int32_t *d_zt = nullptr, *d_wt = nullptr, *d_order = nullptr;
     int32_t *d_slot_beg = nullptr, *d_slot_h = nullptr;
-    double2 *d_gl = nullptr;
+    double2 *d_gl = nullptr, *d_taptab = nullptr;   // quadrature nodes; the taps' cos and sin table
     float *d_cmax = nullptr;          // max(|Re|, |Im|) over the bank (set by jerk_templates)
     int64_t bytes = 0;
     std::atomic<bool> ready{false};   // jerk_templates has filled d_bank
@@ -297,8 +298,7 @@ struct jerk_plan_s {
     int *d_err = nullptr;              // device error flag (bounded waits)
     long long *d_chk = nullptr;        // bounds-check violations and first site (debug build)
     int32_t inject = 0, inject_pos = 0;   // test hook of the debug build (jerk_check_inject)
-    double2 *d_gl = nullptr;
-    int n_gl = 0;
+    double2 *d_gl = nullptr, *d_taptab = nullptr;
     int64_t bytes = 0;
     std::vector<int32_t> h_slot_beg, h_slot_h;
     // state

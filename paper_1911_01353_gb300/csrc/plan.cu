@@ -27,6 +27,7 @@ BankShare::~BankShare() {
     cudaFree(d_slot_beg);
     cudaFree(d_slot_h);
     cudaFree(d_gl);
+    cudaFree(d_taptab);
     cudaFree(d_cmax);
     if (had) cudaSetDevice(cur);
 }
@@ -869,6 +870,7 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
         TRY(dalloc(&sh->bytes, &sh->d_slot_beg, (size_t)pl->T + 1));
         TRY(dalloc(&sh->bytes, &sh->d_slot_h, (size_t)pl->n_entries));
         TRY(dalloc(&sh->bytes, &sh->d_gl, 64));
+        TRY(dalloc(&sh->bytes, &sh->d_taptab, tap_table_elems(pl->b * pl->M)));
         TRY(dalloc(&sh->bytes, &sh->d_cmax, 1));
         TRY(cudaMemcpy(sh->d_zt, pl->zt.data(), sizeof(int32_t) * pl->T, cudaMemcpyHostToDevice));
         TRY(cudaMemcpy(sh->d_order, pl->order.data(), sizeof(int32_t) * pl->T, cudaMemcpyHostToDevice));
@@ -884,6 +886,8 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
             std::vector<double2> gl(64);
             for (int i = 0; i < 64; ++i) gl[i] = make_double2(x[i], w[i]);
             e = cudaMemcpy(sh->d_gl, gl.data(), sizeof(double2) * 64, cudaMemcpyHostToDevice);
+            TRY(launch_tap_table(sh->d_taptab, sh->d_gl, pl->b, pl->b * pl->M, params->pad_bins, nullptr));
+            TRY(cudaStreamSynchronize(nullptr));     // any stream may read the table from here
         }
     }
     if (e == cudaSuccess) {
@@ -896,7 +900,7 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
         pl->d_slot_h = sh->d_slot_h;
         pl->d_gl = sh->d_gl;
         pl->d_cmax = sh->d_cmax;
-        pl->n_gl = 64;
+        pl->d_taptab = sh->d_taptab;
     }
     if (params->precision != 0 && e == cudaSuccess) {
         const std::vector<unsigned char> c = tc_constants(params->precision);
@@ -1078,7 +1082,7 @@ jerk_status jerk_taps(jerk_plan pl, int32_t t0, int32_t nt, void *d_out, void *s
     JCHECK(cudaSetDevice(pl->device));
     cudaStream_t st = (cudaStream_t)stream;
     JCHECK(launch_taps(pl->d_zt, pl->d_wt, nullptr, t0, nt, pl->b, pl->prm.pad_bins, pl->b * pl->M, pl->d_gl,
-                       pl->n_gl, (double2 *)d_out, st));
+                       pl->d_taptab, (double2 *)d_out, st));
     return JERK_OK;
 }
 
@@ -1086,40 +1090,48 @@ jerk_status jerk_templates(jerk_plan pl, void *stream) {
     if (!pl) return JERK_EINVAL;
     JCHECK(cudaSetDevice(pl->device));
     cudaStream_t st = (cudaStream_t)stream;
-    // per bank row (processing order): tap offset shift and filter length of its group
-    std::vector<int32_t> shift(pl->T), klen(pl->T);
+    // tap offset of every bank row's group
+    std::vector<int32_t> off(pl->T);
     for (const auto &g : pl->groups)
-        for (int k = g.tb; k < g.te; ++k) {
-            shift[k] = pl->b * pl->M - g.bM;
-            klen[k] = 2 * g.bM + 1;
+        for (int k = g.tb; k < g.te; ++k) off[k] = g.bM;
+    // the templates with z, w >= 0 and, for each, the bank rows of (+-z, +-w) and their offsets
+    std::vector<int32_t> base, dest, offs;
+    for (int t = 0; t < pl->T; ++t) {
+        const int z = pl->zt[t], w = pl->wt[t];
+        if (z < 0 || w < 0) continue;
+        base.push_back(t);
+        for (int q = 0; q < 4; ++q) {
+            const bool twin = ((q & 1) && z == 0) || ((q & 2) && w == 0);   // the same template again
+            const int row = twin ? -1 : pl->row_of[index_of(pl, (q & 1) ? -z : z, (q & 2) ? -w : w)];
+            dest.push_back(row);
+            offs.push_back(twin ? 0 : off[row]);
         }
-    // process the bank in chunks so the FP64 tap buffer stays small
-    const int chunk = std::max(1, std::min(pl->T, (int)((256u << 20) / ((size_t)pl->K * sizeof(double2)))));
-    double2 *taps = nullptr, *tw = nullptr;
-    int32_t *d_shift = nullptr, *d_klen = nullptr;
-    JCHECK(cudaMallocAsync((void **)&taps, (size_t)chunk * pl->K * sizeof(double2), st));
-    cudaError_t e = cudaMallocAsync((void **)&tw, (size_t)(pl->L / 2) * sizeof(double2), st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void **)&d_shift, sizeof(int32_t) * pl->T, st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void **)&d_klen, sizeof(int32_t) * pl->T, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_shift, shift.data(), sizeof(int32_t) * pl->T, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_klen, klen.data(), sizeof(int32_t) * pl->T, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_twiddles64(tw, pl->L, st);
-    for (int k0 = 0; k0 < pl->T && e == cudaSuccess; k0 += chunk) {
-        const int nt = std::min(chunk, pl->T - k0);
-        e = launch_taps(pl->d_zt, pl->d_wt, pl->d_order + k0, 0, nt, pl->b, pl->prm.pad_bins, pl->b * pl->M,
-                        pl->d_gl, pl->n_gl, taps, st);
-        if (e == cudaSuccess)
-            e = launch_template_fft(taps, d_shift + k0, d_klen + k0, nt, pl->K, pl->L, tw,
-                                    pl->prm.precision ? -kTcBankPair : conv_fold_radix(pl->log2L),
-                                    pl->d_bank + (size_t)k0 * pl->L, st);
     }
-    if (e == cudaSuccess) e = launch_bank_maxabs(pl->d_bank, (int64_t)pl->T * pl->L, pl->d_cmax, pl->sms, st);
-    cudaFreeAsync(taps, st);
-    if (tw) cudaFreeAsync(tw, st);
-    if (d_shift) cudaFreeAsync(d_shift, st);
-    if (d_klen) cudaFreeAsync(d_klen, st);
+    const int nb = (int)base.size();
+    // in chunks, so that the FP64 tap buffer stays within 256 MB
+    const int chunk = std::max(1, std::min(nb, (int)((256u << 20) / ((size_t)pl->K * sizeof(double2)))));
+    const size_t b_taps = align256((size_t)chunk * pl->K * sizeof(double2));
+    const size_t b_tw = align256((size_t)pl->L * sizeof(double2)), b_list = align256(sizeof(int32_t) * nb);
+    char *buf = nullptr;
+    JCHECK(cudaMallocAsync((void **)&buf, b_taps + b_tw + 9 * b_list, st));
+    double2 *taps = (double2 *)buf, *tw = (double2 *)(buf + b_taps);
+    int32_t *d_base = (int32_t *)(buf + b_taps + b_tw);
+    int32_t *d_dest = (int32_t *)((char *)d_base + b_list), *d_offs = (int32_t *)((char *)d_dest + 4 * b_list);
+    cudaError_t e = cudaMemcpyAsync(d_base, base.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_dest, dest.data(), sizeof(int32_t) * 4 * nb, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_offs, offs.data(), sizeof(int32_t) * 4 * nb, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_twiddles64(tw, pl->L, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(pl->d_cmax, 0, sizeof(float), st);
+    for (int k0 = 0; k0 < nb && e == cudaSuccess; k0 += chunk) {
+        const int nt = std::min(chunk, nb - k0);
+        e = launch_taps(pl->d_zt, pl->d_wt, d_base + k0, 0, nt, pl->b, pl->prm.pad_bins, pl->b * pl->M, pl->d_gl,
+                        pl->d_taptab, taps, st);
+        if (e == cudaSuccess)
+            e = launch_template_fft(taps, d_dest + 4 * k0, d_offs + 4 * k0, nt, pl->b * pl->M, pl->L, tw,
+                                    pl->prm.precision ? -kTcBankPair : conv_fold_radix(pl->log2L), pl->d_bank,
+                                    pl->d_cmax, st);
+    }
+    cudaFreeAsync(buf, st);
     // the host vectors above must outlive the copies
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return from_cuda(e);
@@ -1173,7 +1185,7 @@ jerk_status jerk_plane(jerk_plan pl, const void *d_spec, int64_t n, int32_t t0, 
     a.tc_cmax = pl->d_cmax;
     // only the groups that hold a template of the range (a group's positions are
     // in ascending t, so each CTA finds its own by binary search): filtering the
-    // whole bank for 64 of 12 261 templates at 2^18 bins took 12.5 ms
+    // whole bank for 64 of 12 261 templates at 2^18 bins took 12.5 ms, this 0.15 ms
     int64_t first = -1, last = 0, at = 0;
     const int64_t bN = (int64_t)pl->b * n;
     const int segs = conv_segs_per_cta(pl->log2L);
