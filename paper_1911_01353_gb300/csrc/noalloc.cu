@@ -96,25 +96,37 @@ __global__ void __launch_bounds__(kThreads) count_kernel(const unsigned long lon
 
 // 2. exclusive prefix sum of the block counts (one CTA), total into d_count
 __global__ void __launch_bounds__(1024) scan_kernel(unsigned long long *scratch, int nblk, int64_t *d_count) {
-    __shared__ unsigned long long part[1024];
+    __shared__ unsigned long long part[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int per = (nblk + 1023) / 1024;
-    const int b0 = threadIdx.x * per, b1 = min(nblk, b0 + per);
+    const int b0 = min(nblk, (int)threadIdx.x * per), b1 = min(nblk, b0 + per);
     unsigned long long s = 0;
     for (int b = b0; b < b1; ++b) s += scratch[b];
-    part[threadIdx.x] = s;
+    // sums of the threads before this one: within the warp, then over the warps
+    // (one thread adding 1024 parts in turn took most of this kernel's time)
+    unsigned long long incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) part[warp] = incl;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long run = 0;
-        for (int i = 0; i < 1024; ++i) {
-            const unsigned long long v = part[i];
-            part[i] = run;
-            run += v;
+    if (warp == 0) {
+        unsigned long long v = part[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
         }
-        scratch[nblk] = run;
-        *d_count = (int64_t)run;
+        part[lane] = v;
+        if (lane == 31) {
+            scratch[nblk] = v;
+            *d_count = (int64_t)v;
+        }
     }
     __syncthreads();
-    unsigned long long run = part[threadIdx.x];
+    unsigned long long run = incl - s + (warp > 0 ? part[warp - 1] : 0ull);
     for (int b = b0; b < b1; ++b) {
         const unsigned long long v = scratch[b];
         scratch[b] = run;

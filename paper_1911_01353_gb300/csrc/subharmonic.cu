@@ -10,21 +10,49 @@
 // fundamental-indexed sum of the main path adds the same terms where the
 // rounding is exact).
 //
-// One thread per cell q walks the templates in ascending t, adds its H terms
-// in h order in FP32, keeps the running (max, argmax) -- lowest t on equal
-// sums -- and FP64 statistics partials; the plane is read through L2.
+// A block takes 32 consecutive cells: each of its eight warps walks an eighth
+// of the templates for them and the partial (max, argmax) are combined in
+// ascending t (lowest t on equal sums).  The H template indices of every t are
+// a table in shared memory.  A plane of 77 MB is read through L2 at 4 H bytes
+// per sum; with the table, 64-bit divisions no longer come before each load,
+// and eight warps share a cell, so that 2^14 cells already fill the chip.
 #include "jerk_internal.h"
 
 namespace jerk {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kWarps = kThreads / 32;
+constexpr int kTable = 1024;         // templates whose harmonic indices are in shared memory at a time
+constexpr int kFlush = 32;           // sums between two additions to the FP64 statistics
 
+// a h / H to the nearest integer, halves away from zero
 __device__ __forceinline__ int64_t round_ratio(int64_t a, int h, int H) {
     const int64_t m = (a < 0 ? -a : a) * h;
     const int64_t q = (2 * m + H) / (2 * H);
     return a < 0 ? -q : q;
 }
+__device__ __forceinline__ int round_ratio32(int a, int h, int H) {
+    const int q = (2 * abs(a) * h + H) / (2 * H);
+    return a < 0 ? -q : q;
+}
+
+// Sum of FP32 values kept as an unevaluated pair s + c (Knuth's TwoSum: s the
+// rounded sum, c the sum of its exact errors), about 48 bits: FP64 additions run
+// at 1/64 of the FP32 rate here and were the longest part of the sums.
+struct PairSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float y) {
+        const float t = __fadd_rn(s, y);
+        const float b = __fsub_rn(t, s);
+        c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(y, b)));
+        s = t;
+    }
+    __device__ __forceinline__ void flush(double &acc) {
+        acc += (double)s + (double)c;
+        s = c = 0.f;
+    }
+};
 
 struct SubArgs {
     const float *plane;          // [T][bN]
@@ -34,46 +62,104 @@ struct SubArgs {
     double *part;                // [gridDim.x][2] statistics partials
 };
 
+template <int H>
 __global__ void __launch_bounds__(kThreads) subharmonic_kernel(SubArgs a) {
-    __shared__ double r1[kThreads / 32], r2[kThreads / 32];
+    __shared__ int32_t row[kTable][H];
+    __shared__ float smax[kWarps][32];
+    __shared__ int sarg[kWarps][32];
+    __shared__ double r1[kWarps], r2[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double s1 = 0.0, s2 = 0.0;
-    for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < a.bN;
-         q += (int64_t)gridDim.x * kThreads) {
-        int64_t cell[JERK_MAX_HARMONIC];
+    for (int64_t q0 = 32 * (int64_t)blockIdx.x; q0 < a.bN; q0 += 32 * (int64_t)gridDim.x) {
+        const int64_t q = q0 + lane;
+        const bool in = q < a.bN;
+        const float *col[H];
 #pragma unroll
-        for (int h = 1; h <= JERK_MAX_HARMONIC; ++h)
-            if (h <= a.H) cell[h - 1] = round_ratio(q, h, a.H);
+        for (int h = 1; h <= H; ++h) col[h - 1] = a.plane + (in ? round_ratio(q, h, H) : 0);
         float best = -1.0f;
         int bt = 0;
-        for (int t = 0; t < a.T; ++t) {
-            const int zi = t % a.nz - a.zc, wi = t / a.nz - a.wc;
-            float S = 0.0f;
-            for (int h = 1; h <= a.H; ++h) {
-                const int64_t th = (round_ratio(wi, h, a.H) + a.wc) * a.nz + (round_ratio(zi, h, a.H) + a.zc);
-                S += __ldg(a.plane + th * a.bN + cell[h - 1]);
+        for (int tb = 0; tb < a.T; tb += kTable) {
+            const int n = min(kTable, a.T - tb);
+            if (a.T > kTable || q0 == 32 * (int64_t)blockIdx.x) {   // one table serves every cell when it holds all
+                __syncthreads();
+                for (int i = threadIdx.x; i < n; i += kThreads) {
+                    const int t = tb + i, zi = t % a.nz - a.zc, wi = t / a.nz - a.wc;
+#pragma unroll
+                    for (int h = 1; h <= H; ++h)
+                        row[i][h - 1] = (round_ratio32(wi, h, H) + a.wc) * a.nz + (round_ratio32(zi, h, H) + a.zc);
+                }
+                __syncthreads();
             }
-            s1 += (double)S;
-            s2 += (double)S * (double)S;
-            if (S > best) {
-                best = S;
-                bt = t;
+            // this warp's part, ascending; parts and tables ascend too
+            const int i1 = (int)((int64_t)n * (warp + 1) / kWarps);
+            PairSum p1, p2;
+            int k = 0;
+            float pb = -1.0f;
+            int pt = 0;
+#pragma unroll 4
+            for (int i = (int)((int64_t)n * warp / kWarps); i < i1; ++i) {
+                float S = 0.0f;
+#pragma unroll
+                for (int h = 0; h < H; ++h) S += __ldg(col[h] + (int64_t)row[i][h] * a.bN);
+                if (S > pb) {
+                    pb = S;
+                    pt = tb + i;
+                }
+                // S and S^2 as exact pairs in the range where both are normal numbers, else in FP64
+                if (S == 0.0f || (S >= 1e-12f && S <= 1e15f)) {
+                    p1.add(S);
+                    const float sq = __fmul_rn(S, S);
+                    p2.add(sq);
+                    p2.c = __fadd_rn(p2.c, __fmaf_rn(S, S, -sq));
+                } else if (in) {
+                    s1 += (double)S;
+                    s2 += (double)S * (double)S;
+                }
+                if (++k == kFlush) {
+                    k = 0;
+                    if (in) {
+                        p1.flush(s1);
+                        p2.flush(s2);
+                    } else {
+                        p1 = PairSum();
+                        p2 = PairSum();
+                    }
+                }
             }
+            if (in) {
+                p1.flush(s1);
+                p2.flush(s2);
+            }
+            smax[warp][lane] = pb;
+            sarg[warp][lane] = pt;
+            __syncthreads();
+            if (warp == 0) {
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w)
+                    if (smax[w][lane] > best) {
+                        best = smax[w][lane];
+                        bt = sarg[w][lane];
+                    }
+            }
+            __syncthreads();
         }
-        a.M[q] = ((unsigned long long)__float_as_uint(best) << 32) | (unsigned long long)(0xFFFFFFFFu - (unsigned)bt);
+        if (warp == 0 && in)
+            a.M[q] = ((unsigned long long)__float_as_uint(best) << 32) |
+                     (unsigned long long)(0xFFFFFFFFu - (unsigned)bt);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         s1 += __shfl_xor_sync(0xffffffffu, s1, o);
         s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     }
-    if ((threadIdx.x & 31) == 0) {
-        r1[threadIdx.x >> 5] = s1;
-        r2[threadIdx.x >> 5] = s2;
+    if (lane == 0) {
+        r1[warp] = s1;
+        r2[warp] = s2;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         double x1 = 0.0, x2 = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) {
+        for (int w = 0; w < kWarps; ++w) {
             x1 += r1[w];
             x2 += r2[w];
         }
@@ -82,17 +168,43 @@ __global__ void __launch_bounds__(kThreads) subharmonic_kernel(SubArgs a) {
     }
 }
 
-// the partials in block order (deterministic) into sums[0..1]
-__global__ void sum_partials_kernel(const double *part, int n, double *sums) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double x1 = 0.0, x2 = 0.0;
-        for (int i = 0; i < n; ++i) {
-            x1 += part[2 * i];
-            x2 += part[2 * i + 1];
-        }
-        sums[0] = x1;
-        sums[1] = x2;
+// the partials in a fixed order (deterministic) into sums[0..1]
+__global__ void __launch_bounds__(kThreads) sum_partials_kernel(const double *part, int n, double *sums) {
+    __shared__ double r[2][kWarps];
+    double x1 = 0.0, x2 = 0.0;
+    for (int i = threadIdx.x; i < n; i += kThreads) {
+        x1 += part[2 * i];
+        x2 += part[2 * i + 1];
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        x1 += __shfl_xor_sync(0xffffffffu, x1, o);
+        x2 += __shfl_xor_sync(0xffffffffu, x2, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        r[0][threadIdx.x >> 5] = x1;
+        r[1][threadIdx.x >> 5] = x2;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double x = 0.0;
+        for (int w = 0; w < kWarps; ++w) x += r[threadIdx.x][w];
+        sums[threadIdx.x] = x;
+    }
+}
+
+cudaError_t launch_subharmonic(const SubArgs &a, int nblk, cudaStream_t st) {
+    switch (a.H) {
+        case 1: subharmonic_kernel<1><<<nblk, kThreads, 0, st>>>(a); break;
+        case 2: subharmonic_kernel<2><<<nblk, kThreads, 0, st>>>(a); break;
+        case 3: subharmonic_kernel<3><<<nblk, kThreads, 0, st>>>(a); break;
+        case 4: subharmonic_kernel<4><<<nblk, kThreads, 0, st>>>(a); break;
+        case 5: subharmonic_kernel<5><<<nblk, kThreads, 0, st>>>(a); break;
+        case 6: subharmonic_kernel<6><<<nblk, kThreads, 0, st>>>(a); break;
+        case 7: subharmonic_kernel<7><<<nblk, kThreads, 0, st>>>(a); break;
+        default: subharmonic_kernel<8><<<nblk, kThreads, 0, st>>>(a); break;
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -116,12 +228,12 @@ extern "C" jerk_status jerk_subharmonic(jerk_plan pl, const float *d_plane, int6
     a.wc = pl->prm.wmax / pl->prm.dw;
     a.M = (unsigned long long *)d_maxproj;
     a.part = pl->d_stat_part;
-    int64_t nblk = (a.bN + kThreads - 1) / kThreads;
+    int64_t nblk = (a.bN + 31) / 32;
     nblk = std::min<int64_t>(nblk, (int64_t)pl->sms * 8);
     nblk = std::min<int64_t>(nblk, pl->stat_part_cap / 2);
     if (nblk < 1) return JERK_ENOMEM;
-    subharmonic_kernel<<<(unsigned)nblk, kThreads, 0, st>>>(a);
-    sum_partials_kernel<<<1, 32, 0, st>>>(pl->d_stat_part, (int)nblk, d_sums);
+    if (launch_subharmonic(a, (int)nblk, st) != cudaSuccess) return JERK_ECUDA;
+    sum_partials_kernel<<<1, kThreads, 0, st>>>(pl->d_stat_part, (int)nblk, d_sums);
     if (cudaGetLastError() != cudaSuccess) return JERK_ECUDA;
     if (cudaEventRecord(pl->done, st) != cudaSuccess) return JERK_ECUDA;
     return JERK_OK;

@@ -287,33 +287,35 @@ class Plan:
         plane = torch.empty((T, bN), dtype=torch.float32, device=dev)
         self.plane(spec, 0, T, plane, stream=stream)
         p = self.params
-        recs, stats, maxprojs = [], [], []
-        for si in range(int(p.n_stages)):
-            H = int(p.stages[si])
-            M = torch.empty(bN, dtype=torch.int64, device=dev)
-            sums = torch.zeros(2, dtype=torch.float64, device=dev)
-            _check(lib().jerk_subharmonic(self._h, ctypes.c_void_p(plane.data_ptr()), n, H,
-                                          ctypes.c_void_p(M.data_ptr()), ctypes.c_void_p(sums.data_ptr()),
+        H = [int(p.stages[si]) for si in range(int(p.n_stages))]
+        # every stage's sums are enqueued before the first is waited for, then every stage's peaks
+        maxprojs = [torch.empty(bN, dtype=torch.int64, device=dev) for _ in H]
+        sums = torch.empty((len(H), 2), dtype=torch.float64, device=dev)
+        for si, h in enumerate(H):
+            _check(lib().jerk_subharmonic(self._h, ctypes.c_void_p(plane.data_ptr()), n, h,
+                                          ctypes.c_void_p(maxprojs[si].data_ptr()),
+                                          ctypes.c_void_p(sums[si].data_ptr()),
                                           _stream_handle(stream)), "jerk_subharmonic")
-            torch.cuda.synchronize(self.device)
-            s1, s2 = (float(x) for x in sums.cpu())
-            cnt = float(T) * float(bN)
+        torch.cuda.synchronize(self.device)
+        recs, stats = [], []
+        cnt = float(T) * float(bN)
+        size = CANDIDATE_DTYPE.itemsize
+        out = torch.empty((len(H), cap * size), dtype=torch.uint8, device=dev)
+        cnt_d = torch.empty(len(H), dtype=torch.int64, device=dev)
+        for si, (s1, s2) in enumerate(sums.cpu().tolist()):
             mu = s1 / cnt
             sd = math.sqrt(max(0.0, s2 / cnt - mu * mu))
             theta = float(np.float32(mu + float(p.thresh[si]) * sd)) if p.thresh_mode == THRESH_SIGMA \
                 else float(np.float32(p.thresh[si]))
-            out = torch.zeros(cap * CANDIDATE_DTYPE.itemsize, dtype=torch.uint8, device=dev)
-            cnt_d = torch.zeros(1, dtype=torch.int64, device=dev)
-            peaks_noalloc(M.data_ptr(), bN, theta, H, int(p.zmax), int(p.dz), int(p.wmax), int(p.dw),
-                          out.data_ptr(), cap, cnt_d.data_ptr(), stream)
-            torch.cuda.synchronize(self.device)
-            k = int(cnt_d.item())
+            peaks_noalloc(maxprojs[si].data_ptr(), bN, theta, H[si], int(p.zmax), int(p.dz), int(p.wmax), int(p.dw),
+                          out[si].data_ptr(), cap, cnt_d[si:].data_ptr(), stream)
+            stats.append((mu, sd, theta))
+        torch.cuda.synchronize(self.device)
+        for si, k in enumerate(cnt_d.cpu().tolist()):
             if k > cap:
                 raise JerkError(JERK_EOVERFLOW, "jerk_peaks_noalloc (%d found)" % k)
-            raw = out[: k * CANDIDATE_DTYPE.itemsize].cpu().numpy()
+            raw = out[si, : k * size].cpu().numpy()
             recs.extend(np.frombuffer(raw.tobytes(), dtype=CANDIDATE_DTYPE).tolist())
-            stats.append((mu, sd, theta))
-            maxprojs.append(M)
         return recs, stats, maxprojs
 
     def share(self, params: Params) -> "Plan":
