@@ -167,7 +167,19 @@ struct PeakArgs {
     unsigned long long *count;
 };
 
+// spectra of one normalisation launch (by value: the caller's pointers)
+constexpr int kNormItems = 32;
+struct NormArgs {
+    const float2 *in[kNormItems];
+    float2 *out[kNormItems];
+    int64_t n[kNormItems];
+    int32_t blk0[kNormItems];              // first block of each
+    int32_t count;
+};
+
 // launchers (return cudaGetLastError())
+cudaError_t launch_normalise(const float2 *const *in, float2 *const *out, const int64_t *n, int count, int block,
+                             cudaStream_t st);
 cudaError_t launch_normalise(const float2 *in, float2 *out, int64_t n, int block, cudaStream_t st);
 size_t tap_table_elems(int bM);
 cudaError_t launch_tap_table(double2 *tab, const double2 *gl, int b, int bM, int pad, cudaStream_t st);

@@ -9,55 +9,167 @@ namespace jerk {
 // ---------------------------------------------------------------------------
 // Power normalisation (the paper is silent; reading): for each block of B
 // bins, med = element of rank floor((n-1)/2) of |F_k|^2 (FP64, exact for
-// FP32 input), F_k <- F_k (med / ln 2)^(-1/2).  One CTA per block; bitonic
-// sort of the FP64 bit patterns (non-negative, so integer order = value order).
+// FP32 input), F_k <- F_k (med / ln 2)^(-1/2).
+//
+// One warp per block of up to 1024 bins (four warps above), every bin's power
+// rounded to FP32 in a register: rounding keeps the order, so bisecting the
+// FP32 bit patterns by counting (one compare per bin and step, one warp
+// reduction, no barrier) closes in on the powers around the median, and the
+// FP64 powers decide among those that are left, one as a rule after 15 to 20
+// steps.  What bounds it is the FP64 pipe (8 operations and conversions per
+// bin); the bitonic sort of all FP64 powers that this replaces spent 55
+// barriers per block: 2^21 bins 170 -> 89 us, a batch of 24 spectra of 2^13-2^16
+// bins 555 -> 40 us (one launch normalises up to kNormItems spectra).
 // ---------------------------------------------------------------------------
-__global__ void normalise_kernel(const float2 *__restrict__ in, float2 *__restrict__ out, int64_t n,
-                                 int B, int SZ) {
-    extern __shared__ unsigned long long key[];   // [SZ]
-    const int64_t s0 = (int64_t)blockIdx.x * B;
+__device__ __forceinline__ unsigned long long power_key(float2 f) {
+    const double re = f.x, im = f.y;
+    return (unsigned long long)__double_as_longlong(re * re + im * im);   // non-negative: integer order = value order
+}
+
+// sums and extrema over the W warps of a block of bins
+template <int W>
+struct BlockOf {
+    static __device__ __forceinline__ unsigned add(unsigned x) {
+        x = __reduce_add_sync(0xffffffffu, x);
+        if constexpr (W > 1) x = across(x, [](unsigned a, unsigned b) { return a + b; });
+        return x;
+    }
+    static __device__ __forceinline__ unsigned low(unsigned x) {
+        x = __reduce_min_sync(0xffffffffu, x);
+        if constexpr (W > 1) x = across(x, [](unsigned a, unsigned b) { return a < b ? a : b; });
+        return x;
+    }
+    static __device__ __forceinline__ unsigned high(unsigned x) {
+        x = __reduce_max_sync(0xffffffffu, x);
+        if constexpr (W > 1) x = across(x, [](unsigned a, unsigned b) { return a > b ? a : b; });
+        return x;
+    }
+    template <class Op>
+    static __device__ __forceinline__ unsigned across(unsigned x, Op op) {
+        __shared__ unsigned part[W];
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
+        __syncthreads();
+        unsigned r = part[0];
+#pragma unroll
+        for (int w = 1; w < W; ++w) r = op(r, part[w]);
+        __syncthreads();
+        return r;
+    }
+    // a 64-bit minimum or maximum, high word first
+    static __device__ __forceinline__ unsigned long long low64(unsigned long long x) {
+        const unsigned h = low((unsigned)(x >> 32));
+        const unsigned l = low((unsigned)(x >> 32) == h ? (unsigned)x : ~0u);
+        return ((unsigned long long)h << 32) | l;
+    }
+    static __device__ __forceinline__ unsigned long long high64(unsigned long long x) { return ~low64(~x); }
+};
+
+// KPT bins per thread, W warps per block of at most 32 W KPT bins
+template <int KPT, int W>
+__global__ void __launch_bounds__(32 * W) normalise_kernel(NormArgs a, int B) {
+    constexpr int NT = 32 * W;
+    int item = 0;
+    while (item + 1 < a.count && (int)blockIdx.x >= a.blk0[item + 1]) ++item;
+    const int64_t s0 = (int64_t)((int)blockIdx.x - a.blk0[item]) * B, n = a.n[item];
     const int nb = (int)((n - s0) < B ? (n - s0) : B);
-    for (int i = threadIdx.x; i < SZ; i += blockDim.x) {
-        unsigned long long k = ~0ull;
-        if (i < nb) {
-            const float2 f = in[s0 + i];
-            const double re = f.x, im = f.y;
-            k = (unsigned long long)__double_as_longlong(re * re + im * im);
-        }
-        key[i] = k;
-    }
-    __syncthreads();
-    for (int k = 2; k <= SZ; k <<= 1) {
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            for (int i = threadIdx.x; i < SZ; i += blockDim.x) {
-                const int ixj = i ^ jj;
-                if (ixj > i) {
-                    const unsigned long long a = key[i], b = key[ixj];
-                    const bool up = (i & k) == 0;
-                    if ((a > b) == up) {
-                        key[i] = b;
-                        key[ixj] = a;
-                    }
-                }
-            }
-            __syncthreads();
+    const float2 *in = a.in[item] + s0;
+    float2 *out = a.out[item] + s0;
+    const int tid = threadIdx.x;
+    unsigned key[KPT];
+    unsigned lo = ~0u, hi = 0u;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        const int k = tid + NT * i;
+        key[i] = ~0u;                                         // above every power: never counted
+        if (k < nb) {
+            key[i] = __float_as_uint((float)__longlong_as_double((long long)power_key(in[k])));
+            lo = min(lo, key[i]);
+            hi = max(hi, key[i]);
         }
     }
-    const double med = __longlong_as_double((long long)key[(nb - 1) / 2]);
+    lo = BlockOf<W>::low(lo);
+    hi = BlockOf<W>::high(hi);
+    // the median is one of the n_hi - n_lo powers in [lo, hi]
+    const unsigned rank = (unsigned)(nb - 1) / 2;
+    unsigned n_lo = 0, n_hi = (unsigned)nb;
+    while (lo < hi && n_hi - n_lo > 1) {
+        const unsigned mid = lo + (hi - lo) / 2;
+        unsigned c = 0;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) c += key[i] <= mid ? 1u : 0u;
+        c = BlockOf<W>::add(c);
+        if (c > rank) {
+            hi = mid;
+            n_hi = c;
+        } else {
+            lo = mid + 1;
+            n_lo = c;
+        }
+    }
+    // among them, by FP64 powers: their range, then by counting again if it is wider than one value
+    unsigned long long lo64 = ~0ull, hi64 = 0ull;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        if (key[i] >= lo && key[i] <= hi) {
+            const unsigned long long v = power_key(in[tid + NT * i]);
+            lo64 = v < lo64 ? v : lo64;
+            hi64 = v > hi64 ? v : hi64;
+        }
+    }
+    lo64 = BlockOf<W>::low64(lo64);
+    hi64 = BlockOf<W>::high64(hi64);
+    while (lo64 < hi64) {
+        const unsigned long long mid = lo64 + (hi64 - lo64) / 2;
+        unsigned c = 0;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+            if (key[i] >= lo && key[i] <= hi) c += power_key(in[tid + NT * i]) <= mid ? 1u : 0u;
+        c = BlockOf<W>::add(c);
+        if (c > rank - n_lo)
+            hi64 = mid;
+        else
+            lo64 = mid + 1;
+    }
+    const double med = __longlong_as_double((long long)lo64);
     const double scale = med > 0.0 ? 1.0 / sqrt(med / 0.69314718055994530942) : 1.0;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        const float2 f = in[s0 + i];
-        out[s0 + i] = make_float2((float)((double)f.x * scale), (float)((double)f.y * scale));
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        const int k = tid + NT * i;
+        if (k < nb) {
+            const float2 f = in[k];
+            out[k] = make_float2((float)((double)f.x * scale), (float)((double)f.y * scale));
+        }
     }
 }
 
+cudaError_t launch_normalise(const float2 *const *in, float2 *const *out, const int64_t *n, int count, int B,
+                             cudaStream_t st) {
+    for (int i0 = 0; i0 < count; i0 += kNormItems) {
+        NormArgs a;
+        a.count = count - i0 < kNormItems ? count - i0 : kNormItems;
+        int64_t blk = 0;
+        for (int i = 0; i < a.count; ++i) {
+            a.in[i] = in[i0 + i];
+            a.out[i] = out[i0 + i];
+            a.n[i] = n[i0 + i];
+            a.blk0[i] = (int32_t)blk;
+            blk += (n[i0 + i] + B - 1) / B;
+        }
+        if (blk > INT32_MAX) return cudaErrorInvalidValue;
+        if (B <= 256)
+            normalise_kernel<8, 1><<<(unsigned)blk, 32, 0, st>>>(a, B);
+        else if (B <= 1024)
+            normalise_kernel<32, 1><<<(unsigned)blk, 32, 0, st>>>(a, B);
+        else
+            normalise_kernel<32, 4><<<(unsigned)blk, 128, 0, st>>>(a, B);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_normalise(const float2 *in, float2 *out, int64_t n, int B, cudaStream_t st) {
-    int SZ = 1;
-    while (SZ < B) SZ <<= 1;
-    const int64_t nblk = (n + B - 1) / B;
-    const size_t sm = (size_t)SZ * sizeof(unsigned long long);
-    normalise_kernel<<<(unsigned)nblk, 512, sm, st>>>(in, out, n, B, SZ);
-    return cudaGetLastError();
+    return launch_normalise(&in, &out, &n, 1, B, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -610,12 +610,14 @@ jerk_status enqueue_search(jerk_plan_s *pl, const float2 *const *in, cudaStream_
     const bool sigma = pl->prm.thresh_mode == JERK_THRESH_SIGMA;
 
     JCHECK(mark(pl, 0, st, capturing));
-    for (int i = 0; i < count; ++i) {
-        float2 *dst = pl->d_spec_norm + L.spec_off[i];
-        if (pl->prm.norm_block > 0)
-            JCHECK(launch_normalise(in[i], dst, L.n[i], pl->prm.norm_block, st));
-        else if (in[i] != dst)
-            JCHECK(cudaMemcpyAsync(dst, in[i], sizeof(float2) * L.n[i], cudaMemcpyDeviceToDevice, st));
+    std::vector<float2 *> dst(count);
+    for (int i = 0; i < count; ++i) dst[i] = pl->d_spec_norm + L.spec_off[i];
+    if (pl->prm.norm_block > 0) {
+        JCHECK(launch_normalise(in, dst.data(), L.n.data(), count, pl->prm.norm_block, st));
+    } else {
+        for (int i = 0; i < count; ++i)
+            if (in[i] != dst[i])
+                JCHECK(cudaMemcpyAsync(dst[i], in[i], sizeof(float2) * L.n[i], cudaMemcpyDeviceToDevice, st));
     }
     for (int si = 0; si < ns; ++si) {
         const int64_t used = L.m_off[si][count - 1] + n_cells((int64_t)pl->b * L.n[count - 1], pl->prm.stages[si]);
