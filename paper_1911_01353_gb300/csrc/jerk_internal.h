@@ -46,6 +46,13 @@ struct ItemDesc {
     unsigned long long *M1;  // stage-1 max-projection of this spectrum
     const int64_t *slot_off; // [n_entries] harmonic-row offsets of this spectrum (floats)
     const int64_t *slot_len; // [n_entries] harmonic-row lengths
+    // harmonic sums, statistics and peaks (one launch of each serves every item)
+    const FundEntry *fund;   // fundamentals of stages > 1
+    int64_t n_cells[JERK_MAX_STAGES];
+    unsigned long long *M[JERK_MAX_STAGES];
+    int64_t cta0, n_ctas;    // conv CTAs whose statistics count
+    int64_t harm0;           // first harmonic block
+    int32_t n_fund, harm_nx, harm_ny;   // harmonic blocks: harm_nx of cells by harm_ny of fundamentals
 };
 
 // Arguments of the fused overlap-and-save kernel.
@@ -142,28 +149,28 @@ static_assert(offsetof(RowEntries, off) % 8 == 0 && offsetof(RowEntries, len) % 
 static_assert(sizeof(TplMeta) == 16 && offsetof(TplMeta, e0) % 4 == 0, "TplMeta layout");
 
 struct HarmArgs {
+    const ItemDesc *items;
     const float *slots;
-    const FundEntry *fund;
-    int32_t n_fund;
-    int32_t n_stages;
+    int32_t n_items, n_stages;
     int32_t stages[JERK_MAX_STAGES];
-    int64_t n_cells[JERK_MAX_STAGES];     // floor((bN-1)/H) + 1
-    unsigned long long *M[JERK_MAX_STAGES];
-    double *stat_part;                     // [gridDim.x][n_stages][2]
-    int32_t f_chunk;                       // fundamentals per block (y split)
+    double *stat_part;                     // [blocks][n_stages][2]
     int *err;                              // set on an expired wait (JERK_ETIMEOUT)
     int64_t slot_cap;                      // floats of `slots` (bounds checks of the debug build)
     long long *chk;                        // violation counter and first site (debug build)
 };
 
 struct PeakArgs {
-    const unsigned long long *M[JERK_MAX_STAGES];
-    int64_t n_cells[JERK_MAX_STAGES];
-    const float *theta;                    // device, per stage
-    int32_t n_stages;
-    int32_t item;
+    const ItemDesc *items;
+    const float *theta;                    // device, [item][JERK_MAX_STAGES]
     DevCand *out;
     int64_t cap;
+    unsigned long long *count;
+};
+
+// what a search clears before it starts: the max-projections' used parts and the candidate count
+struct ClearArgs {
+    unsigned long long *M[JERK_MAX_STAGES];
+    int64_t n[JERK_MAX_STAGES];
     unsigned long long *count;
 };
 
@@ -195,12 +202,13 @@ cudaError_t launch_twiddles64(double2 *tw, int L, cudaStream_t st);
 cudaError_t launch_conv(int log2L, int mode, bool stats, const ConvArgs &a, int n_ctas, cudaStream_t st);
 cudaError_t launch_conv_tc(int precision, int mode, bool stats, const ConvArgs &a, int n_ctas, cudaStream_t st);
 int conv_segs_per_cta(int log2L);
-cudaError_t launch_harmonic(const HarmArgs &a, int nblk_y, bool stats, cudaStream_t st);
+cudaError_t launch_harmonic(const HarmArgs &a, int64_t blocks, bool stats, cudaStream_t st);
 int harmonic_cells_per_block();
-cudaError_t launch_finalise_stats(const double *part1, int64_t n1, const double *partH, int64_t nH,
+cudaError_t launch_finalise_stats(const ItemDesc *items, int n_items, const double *part1, const double *partH,
                                   int n_stages, const double *counts, const float *thresh, int mode,
                                   double *stats_out, float *theta_out, cudaStream_t st);
-cudaError_t launch_peaks(const PeakArgs &a, int sms, cudaStream_t st);
+cudaError_t launch_peaks(const PeakArgs &a, int n_items, int n_stages, int64_t most_cells, int sms, cudaStream_t st);
+cudaError_t launch_clear(const ClearArgs &a, int sms, cudaStream_t st);
 cudaError_t launch_wait_check(int *err, uint64_t limit_ns, cudaStream_t st);
 cudaError_t measure_peaks(int sms, double *fp32_tflops, double *l2_gbs);
 cudaError_t measure_packed_fma(int sms, double *tflops);
@@ -223,7 +231,8 @@ struct BatchLayout {
     int64_t total_ctas = 0;
     int n_work = 0;
     std::vector<int64_t> item_cta0;                // [count + 1] conv CTAs of each item
-    std::vector<int64_t> harm0;                    // [count + 1] harmonic partial blocks of each item
+    std::vector<int64_t> harm0;                    // [count + 1] harmonic blocks before each item
+    std::vector<int32_t> harm_ny;                  // [count] parts of an item's fundamentals
     std::vector<int64_t> spec_off;                 // [count] offset in the normalised-spectrum buffer
     std::vector<int64_t> m_off[JERK_MAX_STAGES];   // [count] offset in each max-projection buffer
     std::vector<int64_t> slot_base;                // [count + 1] harmonic-row floats of each item

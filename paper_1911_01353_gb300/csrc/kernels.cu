@@ -186,7 +186,11 @@ cudaError_t launch_normalise(const float2 *in, float2 *out, int64_t n, int B, cu
 // one lane issues the copies, writing each slot's (t, top stage) beside it.
 // Consumers sum their cells of each row in fixed h order (FP32), keep
 // (max, argmax) per stage (lowest t on ties) and the statistics partials,
-// and release each slot per warp.  Every wait is bounded (about one
+// and release each slot per warp.  One launch serves every spectrum of a
+// batch (24 spectra of 2^13-2^16 bins: 727 -> 68 us); where a spectrum's cells
+// alone would leave SMs idle, its fundamentals are split over several blocks
+// (harm_ny) that meet in an atomic maximum (2^16 bins, 33 fundamentals: 31 ->
+// 14 us).  Every wait is bounded (about one
 // second); on expiry the block sets the error flag and leaves after its
 // copies in flight have landed.
 // ---------------------------------------------------------------------------
@@ -202,7 +206,7 @@ struct HarmEntry {                              // a table entry as the producer
 };
 
 template <int NS>
-__global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a, bool stats) {
+__global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(const __grid_constant__ HarmArgs a, bool stats) {
     extern __shared__ __align__(128) float4 ring[];   // [HR][HC_CELLS / 4]
     __shared__ __align__(8) uint64_t full[HR];        // row chunk landed
     __shared__ __align__(8) uint64_t empty[HR];       // every consumer warp done with the slot
@@ -212,11 +216,23 @@ __global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a
     __shared__ double dacc[NS - 1][2][HC_THREADS];    // per-thread FP64 statistics of stages 1.. (kept out of registers)
     constexpr int Q = HC_CELLS / 4;                   // float4 per slot
     const int tid = threadIdx.x;
-    const int64_t c0 = (int64_t)blockIdx.x * HC_CELLS;
+    // the item of this block, and its cells and fundamentals
+    int lo = 0, hi = a.n_items - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((int64_t)blockIdx.x >= __ldg(&a.items[mid].harm0)) lo = mid; else hi = mid - 1;
+    }
+    const ItemDesc *itm = a.items + lo;
+    const int local = (int)((int64_t)blockIdx.x - __ldg(&itm->harm0));
+    const int nx = __ldg(&itm->harm_nx), ny = __ldg(&itm->harm_ny);
+    const int64_t c0 = (int64_t)(local % nx) * HC_CELLS;
+    __shared__ int64_t n_cells[NS];
+    if (tid < NS) n_cells[tid] = __ldg(&itm->n_cells[tid]);
+    __syncthreads();
     int topb = 0;   // highest stage index with cells in this block
 #pragma unroll
     for (int si = 1; si < NS; ++si)
-        if (c0 < a.n_cells[si]) topb = si;
+        if (c0 < n_cells[si]) topb = si;
     int hlo[NS], hhi[NS];
 #pragma unroll
     for (int si = 1; si < NS; ++si) {
@@ -228,8 +244,11 @@ __global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a
         mbar_init(&empty[tid], HC_THREADS / 32);
     }
     __syncthreads();
-    const int f0 = blockIdx.y * a.f_chunk;
-    const int f1 = min(a.n_fund, f0 + a.f_chunk);
+    const int n_fund = __ldg(&itm->n_fund);
+    const int part = local / nx;
+    const int f0 = (int)((int64_t)n_fund * part / ny), f1 = (int)((int64_t)n_fund * (part + 1) / ny);
+    const FundEntry *fund = reinterpret_cast<const FundEntry *>(
+        __ldg(reinterpret_cast<const unsigned long long *>(&itm->fund)));
 
     if (tid >= HC_THREADS) {
         // ---- producer warp ----
@@ -237,7 +256,7 @@ __global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a
         uint32_t bytes[NS];   // chunk bytes of a stage-si row: rows hold n_cells[si] cells, padded to 32
 #pragma unroll
         for (int si = 1; si < NS; ++si) {
-            const int64_t avail = ((a.n_cells[si] + 3) & ~(int64_t)3) - c0;
+            const int64_t avail = ((n_cells[si] + 3) & ~(int64_t)3) - c0;
             bytes[si] = (uint32_t)(4 * (avail < HC_CELLS ? (avail > 0 ? avail : 0) : HC_CELLS));
         }
         int slot = 0, round = 0, issued = 0;
@@ -245,7 +264,7 @@ __global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a
         for (int fb = f0; fb < f1 && good; fb += 32) {
             const int f = fb + plane;
             if (f < f1) {
-                const FundEntry *fe = a.fund + f;
+                const FundEntry *fe = fund + f;
                 const int st = min(__ldg(&fe->top_stage), topb);
                 const int H = a.stages[st];
                 tab[plane].t = __ldg(&fe->t);
@@ -318,7 +337,7 @@ __global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a
             c1[si] = c2[si] = 0.f;
         }
         // cell of (u, c): p0 + 4 HC_THREADS u + c
-        auto cell_ok = [&](int si, int k) { return p0 + 4 * HC_THREADS * (k >> 2) + (k & 3) < a.n_cells[si]; };
+        auto cell_ok = [&](int si, int k) { return p0 + 4 * HC_THREADS * (k >> 2) + (k & 3) < n_cells[si]; };
         if (topb > 0) {
             int slot = 0, cnt = 0;
             uint32_t phase = 0;
@@ -397,11 +416,11 @@ __global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a
                             const unsigned long long packed =
                                 ((unsigned long long)__float_as_uint(mx[si][c]) << 32) |
                                 (unsigned long long)(0xFFFFFFFFu - (unsigned)am[si][c]);
-                            if (!JERK_CHECK(p < a.n_cells[si], a.chk, kChkHarmStore)) continue;
-                            if (gridDim.y == 1)
-                                a.M[si][p] = packed;
+                            if (!JERK_CHECK(p < n_cells[si], a.chk, kChkHarmStore)) continue;
+                            if (ny == 1)
+                                itm->M[si][p] = packed;
                             else
-                                atomicMax(a.M[si] + p, packed);
+                                atomicMax(itm->M[si] + p, packed);
                         }
                     }
                 }
@@ -426,7 +445,7 @@ __global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a
     }
     __syncthreads();
     if (stats && tid == 0) {
-        const int64_t blk = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
+        const int64_t blk = blockIdx.x;
         for (int si = 1; si < NS; ++si) {
             double s1 = 0.0, s2 = 0.0;
             for (int w = 0; w < HC_THREADS / 32; ++w) {
@@ -440,82 +459,87 @@ __global__ void __launch_bounds__(HC_THREADS + 32, 2) harmonic_kernel(HarmArgs a
 }
 
 template <int NS>
-static cudaError_t launch_harmonic_ns(const HarmArgs &a, dim3 grid, bool stats, cudaStream_t st) {
+static cudaError_t launch_harmonic_ns(const HarmArgs &a, unsigned blocks, bool stats, cudaStream_t st) {
     const int smem = HR * HC_CELLS * (int)sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(harmonic_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    harmonic_kernel<NS><<<grid, HC_THREADS + 32, smem, st>>>(a, stats);
+    harmonic_kernel<NS><<<blocks, HC_THREADS + 32, smem, st>>>(a, stats);
     return cudaGetLastError();
 }
 
 int harmonic_cells_per_block() { return HC_CELLS; }
 
-cudaError_t launch_harmonic(const HarmArgs &a, int nblk_y, bool stats, cudaStream_t st) {
-    const int64_t nblk = (a.n_cells[1] + HC_CELLS - 1) / HC_CELLS;
-    const dim3 grid((unsigned)nblk, (unsigned)nblk_y);
+cudaError_t launch_harmonic(const HarmArgs &a, int64_t blocks, bool stats, cudaStream_t st) {
+    if (blocks > INT32_MAX) return cudaErrorInvalidValue;
     switch (a.n_stages) {
-        case 2: return launch_harmonic_ns<2>(a, grid, stats, st);
-        case 3: return launch_harmonic_ns<3>(a, grid, stats, st);
-        case 4: return launch_harmonic_ns<4>(a, grid, stats, st);
+        case 2: return launch_harmonic_ns<2>(a, (unsigned)blocks, stats, st);
+        case 3: return launch_harmonic_ns<3>(a, (unsigned)blocks, stats, st);
+        case 4: return launch_harmonic_ns<4>(a, (unsigned)blocks, stats, st);
         default: return cudaErrorInvalidValue;
     }
 }
 
 // ---------------------------------------------------------------------------
 // Statistics (Sec. 3: mean and standard deviation) -> thresholds.  Partial
-// sums are reduced in a fixed order, so the result is deterministic.
+// sums are reduced in a fixed order, so the result is deterministic.  One
+// block per (item, stage).
 // ---------------------------------------------------------------------------
-__global__ void finalise_stats_kernel(const double *part1, int64_t n1, const double *partH, int64_t nH,
+__global__ void finalise_stats_kernel(const ItemDesc *items, const double *part1, const double *partH,
                                       int n_stages, const double *counts, const float *thresh, int mode,
                                       double *stats_out, float *theta_out) {
     __shared__ double r1[256], r2[256];
-    for (int si = 0; si < n_stages; ++si) {
-        double s1 = 0.0, s2 = 0.0;
-        if (mode == JERK_THRESH_SIGMA) {
-            if (si == 0) {
-                for (int64_t i = threadIdx.x; i < n1; i += blockDim.x) {
-                    s1 += part1[2 * i];
-                    s2 += part1[2 * i + 1];
-                }
-            } else {
-                for (int64_t i = threadIdx.x; i < nH; i += blockDim.x) {
-                    s1 += partH[(i * n_stages + si) * 2];
-                    s2 += partH[(i * n_stages + si) * 2 + 1];
-                }
+    const int si = blockIdx.x, item = blockIdx.y;
+    const ItemDesc *itm = items + item;
+    double s1 = 0.0, s2 = 0.0;
+    if (mode == JERK_THRESH_SIGMA) {
+        if (si == 0) {
+            const double *p = part1 + 2 * itm->cta0;
+            const int64_t n = itm->n_ctas;
+            for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+                s1 += p[2 * i];
+                s2 += p[2 * i + 1];
+            }
+        } else {
+            const double *p = partH + 2 * n_stages * itm->harm0;
+            const int64_t n = (int64_t)itm->harm_nx * itm->harm_ny;
+            for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+                s1 += p[(i * n_stages + si) * 2];
+                s2 += p[(i * n_stages + si) * 2 + 1];
             }
         }
-        r1[threadIdx.x] = s1;
-        r2[threadIdx.x] = s2;
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o) {
-                r1[threadIdx.x] += r1[threadIdx.x + o];
-                r2[threadIdx.x] += r2[threadIdx.x + o];
-            }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            double mu = 0.0, sd = 0.0;
-            float theta = thresh[si];
-            if (mode == JERK_THRESH_SIGMA && counts[si] > 0.0) {
-                mu = r1[0] / counts[si];
-                const double var = r2[0] / counts[si] - mu * mu;
-                sd = sqrt(var > 0.0 ? var : 0.0);
-                theta = (float)(mu + (double)thresh[si] * sd);
-            }
-            stats_out[2 * si] = mu;
-            stats_out[2 * si + 1] = sd;
-            theta_out[si] = theta;
+    }
+    r1[threadIdx.x] = s1;
+    r2[threadIdx.x] = s2;
+    __syncthreads();
+    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) {
+            r1[threadIdx.x] += r1[threadIdx.x + o];
+            r2[threadIdx.x] += r2[threadIdx.x + o];
         }
         __syncthreads();
     }
+    if (threadIdx.x == 0) {
+        const double cnt = counts[item * JERK_MAX_STAGES + si];
+        double mu = 0.0, sd = 0.0;
+        float theta = thresh[si];
+        if (mode == JERK_THRESH_SIGMA && cnt > 0.0) {
+            mu = r1[0] / cnt;
+            const double var = r2[0] / cnt - mu * mu;
+            sd = sqrt(var > 0.0 ? var : 0.0);
+            theta = (float)(mu + (double)thresh[si] * sd);
+        }
+        stats_out[2 * (item * JERK_MAX_STAGES + si)] = mu;
+        stats_out[2 * (item * JERK_MAX_STAGES + si) + 1] = sd;
+        theta_out[item * JERK_MAX_STAGES + si] = theta;
+    }
 }
 
-cudaError_t launch_finalise_stats(const double *part1, int64_t n1, const double *partH, int64_t nH,
+cudaError_t launch_finalise_stats(const ItemDesc *items, int n_items, const double *part1, const double *partH,
                                   int n_stages, const double *counts, const float *thresh, int mode,
                                   double *stats_out, float *theta_out, cudaStream_t st) {
-    finalise_stats_kernel<<<1, 256, 0, st>>>(part1, n1, partH, nH, n_stages, counts, thresh, mode, stats_out,
-                                             theta_out);
+    const dim3 grid((unsigned)n_stages, (unsigned)n_items);
+    finalise_stats_kernel<<<grid, 256, 0, st>>>(items, part1, partH, n_stages, counts, thresh, mode, stats_out,
+                                                theta_out);
     return cudaGetLastError();
 }
 
@@ -528,10 +552,10 @@ cudaError_t launch_finalise_stats(const double *part1, int64_t n1, const double 
 __device__ __forceinline__ float mval(unsigned long long x) { return __uint_as_float((unsigned)(x >> 32)); }
 
 __global__ void peaks_kernel(PeakArgs a) {
-    const int si = blockIdx.y;
-    const int64_t n = a.n_cells[si];
-    const unsigned long long *M = a.M[si];
-    const float theta = a.theta[si];
+    const int si = blockIdx.y, item = blockIdx.z;
+    const int64_t n = a.items[item].n_cells[si];
+    const unsigned long long *M = a.items[item].M[si];
+    const float theta = a.theta[item * JERK_MAX_STAGES + si];
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
          p += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long x = M[p];
@@ -547,21 +571,43 @@ __global__ void peaks_kernel(PeakArgs a) {
                 c.t = (int32_t)(0xFFFFFFFFu - (unsigned)(x & 0xFFFFFFFFull));
                 c.stage_idx = si;
                 c.power = v;
-                c.item = a.item;
+                c.item = item;
                 a.out[idx] = c;
             }
         }
     }
 }
 
-cudaError_t launch_peaks(const PeakArgs &a, int sms, cudaStream_t st) {
-    int64_t nmax = 0;
-    for (int si = 0; si < a.n_stages; ++si) nmax = a.n_cells[si] > nmax ? a.n_cells[si] : nmax;
-    int64_t nblk = (nmax + 255) / 256;
-    if (nblk > (int64_t)sms * 16) nblk = (int64_t)sms * 16;
+cudaError_t launch_peaks(const PeakArgs &a, int n_items, int n_stages, int64_t most_cells, int sms, cudaStream_t st) {
+    int64_t nblk = (most_cells + 255) / 256;
+    const int64_t most = std::max<int64_t>(1, (int64_t)sms * 16 / n_items);   // every item and stage has its own blocks
+    if (nblk > most) nblk = most;
     if (nblk < 1) nblk = 1;
-    dim3 grid((unsigned)nblk, (unsigned)a.n_stages);
+    const dim3 grid((unsigned)nblk, (unsigned)n_stages, (unsigned)n_items);
     peaks_kernel<<<grid, 256, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Everything a search starts from 0, in one launch: the max-projections of
+// all stages (8-byte words, 16 bytes at a time) and the candidate count.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) clear_kernel(ClearArgs a) {
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll
+    for (int si = 0; si < JERK_MAX_STAGES; ++si) {
+        ulonglong2 *M = reinterpret_cast<ulonglong2 *>(a.M[si]);   // its own allocation: 256-byte aligned
+        const int64_t n = a.n[si];
+        for (int64_t i = i0; i < n / 2; i += step) M[i] = make_ulonglong2(0ull, 0ull);
+        if (i0 == 0 && (n & 1)) a.M[si][n - 1] = 0ull;
+    }
+    if (i0 == 0) *a.count = 0ull;
+}
+
+cudaError_t launch_clear(const ClearArgs &a, int sms, cudaStream_t st) {
+    int64_t nblk = (a.n[0] / 2 + 255) / 256;
+    nblk = std::max<int64_t>(1, std::min<int64_t>(nblk, (int64_t)sms * 8));
+    clear_kernel<<<(unsigned)nblk, 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 

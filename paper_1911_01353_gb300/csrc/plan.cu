@@ -218,10 +218,19 @@ int64_t transforms_for(const jerk_plan_s *pl, int64_t n) {
     return s;
 }
 
-int64_t harm_blocks_for(const jerk_plan_s *pl, int64_t n) {
+// Harmonic blocks of a spectrum of n bins: blocks of cells, times parts of its
+// nf fundamentals where the cells alone would leave SMs without a block (a part
+// keeps at least 8 fundamentals).  The split depends on the spectrum alone, so
+// its statistics are added in the same order in every batch.
+int64_t harm_nx_for(const jerk_plan_s *pl, int64_t n) {
     if (pl->prm.n_stages < 2) return 0;
     const int64_t cpb = harmonic_cells_per_block();
     return (n_cells((int64_t)pl->b * n, pl->prm.stages[1]) + cpb - 1) / cpb;
+}
+
+int harm_ny_for(const jerk_plan_s *pl, int64_t nx, int nf) {
+    if (nx < 1) return 1;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(pl->sms / nx, nf / 8));
 }
 
 jerk_status validate(const jerk_params *p) {
@@ -350,6 +359,7 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
     L.total_ctas = 0;
     L.item_cta0.assign(count + 1, 0);
     L.harm0.assign(count + 1, 0);
+    L.harm_ny.assign(count, 1);
     L.spec_off.assign(count, 0);
     L.slot_base.assign(count + 1, 0);
     L.n_fund.assign(count, 0);
@@ -420,7 +430,8 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
             }
         }
         L.item_cta0[i + 1] = L.total_ctas;
-        L.harm0[i + 1] = L.harm0[i] + harm_blocks_for(pl, n[i]);
+        L.harm_ny[i] = harm_ny_for(pl, harm_nx_for(pl, n[i]), nf);
+        L.harm0[i + 1] = L.harm0[i] + harm_nx_for(pl, n[i]) * L.harm_ny[i];
         h.counts[(size_t)i * JERK_MAX_STAGES] = (double)bN * nt_item;
         for (int si = 1; si < ns; ++si)
             h.counts[(size_t)i * JERK_MAX_STAGES + si] = (double)nf_stage[si] * n_cells(bN, pl->prm.stages[si]);
@@ -450,6 +461,17 @@ void fill_items(const jerk_plan_s *pl, const BatchLayout &L, HostTables &h) {
         it.M1 = pl->d_M[0] + L.m_off[0][i];
         it.slot_off = L.d_soff + i * pl->n_entries;
         it.slot_len = L.d_slen + i * pl->n_entries;
+        it.fund = L.d_fund + i * pl->n_fund;
+        for (int si = 0; si < pl->prm.n_stages; ++si) {
+            it.n_cells[si] = n_cells(it.bN, pl->prm.stages[si]);
+            it.M[si] = pl->d_M[si] + L.m_off[si][i];
+        }
+        it.cta0 = L.item_cta0[i];
+        it.n_ctas = L.stat_ctas >= 0 ? L.stat_ctas : L.item_cta0[i + 1] - L.item_cta0[i];
+        it.harm0 = L.harm0[i];
+        it.n_fund = L.n_fund[i];
+        it.harm_nx = (int32_t)harm_nx_for(pl, L.n[i]);
+        it.harm_ny = L.harm_ny[i];
     }
 }
 
@@ -619,10 +641,14 @@ jerk_status enqueue_search(jerk_plan_s *pl, const float2 *const *in, cudaStream_
             if (in[i] != dst[i])
                 JCHECK(cudaMemcpyAsync(dst[i], in[i], sizeof(float2) * L.n[i], cudaMemcpyDeviceToDevice, st));
     }
+    ClearArgs cl;
+    std::memset(&cl, 0, sizeof(cl));
     for (int si = 0; si < ns; ++si) {
-        const int64_t used = L.m_off[si][count - 1] + n_cells((int64_t)pl->b * L.n[count - 1], pl->prm.stages[si]);
-        JCHECK(cudaMemsetAsync(pl->d_M[si], 0, sizeof(unsigned long long) * used, st));
+        cl.M[si] = pl->d_M[si];
+        cl.n[si] = L.m_off[si][count - 1] + n_cells((int64_t)pl->b * L.n[count - 1], pl->prm.stages[si]);
     }
+    cl.count = pl->d_count;
+    JCHECK(launch_clear(cl, pl->sms, st));
     JCHECK(mark(pl, 1, st, capturing));
 
     // fused overlap-and-save + stage-1 max-projection + harmonic rows, all spectra in one launch
@@ -652,43 +678,30 @@ jerk_status enqueue_search(jerk_plan_s *pl, const float2 *const *in, cudaStream_
                              : launch_conv(pl->log2L, 0, sigma, a, (int)L.total_ctas, st));
     JCHECK(mark(pl, 2, st, capturing));
 
-    // harmonic sums for stages > 1, per spectrum
+    // harmonic sums for stages > 1, all spectra in one launch
     double *partH = pl->d_stat_part + 2 * L.total_ctas;
     if (ns > 1) {
-        for (int i = 0; i < count; ++i) {
-            const int64_t bN = (int64_t)pl->b * L.n[i];
-            HarmArgs h;
-            std::memset(&h, 0, sizeof(h));
-            h.slots = pl->d_slots;
-            h.fund = L.d_fund + (size_t)i * pl->n_fund;
-            h.n_fund = L.n_fund[i];
-            h.n_stages = ns;
-            for (int si = 0; si < ns; ++si) {
-                h.stages[si] = pl->prm.stages[si];
-                h.n_cells[si] = n_cells(bN, pl->prm.stages[si]);
-                h.M[si] = pl->d_M[si] + L.m_off[si][i];
-            }
-            h.stat_part = partH + 2 * ns * L.harm0[i];
-            h.f_chunk = L.n_fund[i];
-            h.err = pl->d_err;
-            h.chk = pl->d_chk;
-            h.slot_cap = pl->slot_cap;
-            JCHECK(launch_harmonic(h, 1, sigma, st));
-        }
+        HarmArgs h;
+        std::memset(&h, 0, sizeof(h));
+        h.items = L.d_items;
+        h.slots = pl->d_slots;
+        h.n_items = count;
+        h.n_stages = ns;
+        for (int si = 0; si < ns; ++si) h.stages[si] = pl->prm.stages[si];
+        h.stat_part = partH;
+        h.err = pl->d_err;
+        h.chk = pl->d_chk;
+        h.slot_cap = pl->slot_cap;
+        JCHECK(launch_harmonic(h, L.harm0[count], sigma, st));
     }
     JCHECK(mark(pl, 3, st, capturing));
-    for (int i = 0; i < count; ++i)
-        JCHECK(launch_finalise_stats(pl->d_stat_part + 2 * L.item_cta0[i],
-                                     L.stat_ctas >= 0 ? L.stat_ctas : L.item_cta0[i + 1] - L.item_cta0[i],
-                                     partH + 2 * ns * L.harm0[i], L.harm0[i + 1] - L.harm0[i], ns,
-                                     L.d_counts + (size_t)i * JERK_MAX_STAGES, pl->d_thresh, pl->prm.thresh_mode,
-                                     pl->d_stats + (size_t)i * 2 * JERK_MAX_STAGES,
-                                     pl->d_theta + (size_t)i * JERK_MAX_STAGES, st));
+    JCHECK(launch_finalise_stats(L.d_items, count, pl->d_stat_part, partH, ns, L.d_counts, pl->d_thresh,
+                                 pl->prm.thresh_mode, pl->d_stats, pl->d_theta, st));
 
     // peaks
     JCHECK(mark(pl, 4, st, capturing));
     if (peaks) {
-        const jerk_status ps = enqueue_peaks(pl, st);
+        const jerk_status ps = enqueue_peaks(pl, st);     // (the count is cleared above)
         if (ps != JERK_OK) return ps;
     }
     JCHECK(mark(pl, 5, st, capturing));
@@ -698,25 +711,14 @@ jerk_status enqueue_search(jerk_plan_s *pl, const float2 *const *in, cudaStream_
 // thresholded peaks of every spectrum of the current layout (Sec. 3)
 jerk_status enqueue_peaks(jerk_plan_s *pl, cudaStream_t st) {
     const BatchLayout &L = *pl->cur;
-    const int count = (int)L.n.size();
-    const int ns = pl->prm.n_stages;
-    JCHECK(cudaMemsetAsync(pl->d_count, 0, sizeof(unsigned long long), st));
-    for (int i = 0; i < count; ++i) {
-        const int64_t bN = (int64_t)pl->b * L.n[i];
-        PeakArgs pk;
-        std::memset(&pk, 0, sizeof(pk));
-        for (int si = 0; si < ns; ++si) {
-            pk.M[si] = pl->d_M[si] + L.m_off[si][i];
-            pk.n_cells[si] = n_cells(bN, pl->prm.stages[si]);
-        }
-        pk.theta = pl->d_theta + (size_t)i * JERK_MAX_STAGES;
-        pk.n_stages = ns;
-        pk.item = i;
-        pk.out = pl->d_cand;
-        pk.cap = pl->prm.max_candidates;
-        pk.count = pl->d_count;
-        JCHECK(launch_peaks(pk, pl->sms, st));
-    }
+    PeakArgs pk;
+    pk.items = L.d_items;
+    pk.theta = pl->d_theta;
+    pk.out = pl->d_cand;
+    pk.cap = pl->prm.max_candidates;
+    pk.count = pl->d_count;
+    JCHECK(launch_peaks(pk, (int)L.n.size(), pl->prm.n_stages,
+                        (int64_t)pl->b * *std::max_element(L.n.begin(), L.n.end()), pl->sms, st));
     return JERK_OK;
 }
 
@@ -843,7 +845,9 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
     pl->slot_cap = item_rows(pl, N, params->zmax, params->wmax, 0, nullptr, nullptr, nullptr, nullptr, nullptr) +
                    (int64_t)pl->max_batch * 32 * std::max(1, pl->n_fund * JERK_MAX_HARMONIC);
     const int64_t conv_blocks = ctas_for(pl, N) + (int64_t)pl->max_batch * (int64_t)pl->groups.size();
-    const int64_t harm_blocks = harm_blocks_for(pl, N) + pl->max_batch;
+    // (a spectrum's harmonic blocks are at most one per SM more than its blocks of cells)
+    const int64_t harm_blocks = harm_nx_for(pl, N) + (int64_t)pl->max_batch *
+                                (1 + std::min<int64_t>(pl->sms, (int64_t)(pl->n_fund / 8 + 1) * (harm_nx_for(pl, N) + 1)));
     // (a partial search by template range runs each group's templates of the range
     // and, separately, the other templates its fundamentals need: up to twice the CTAs)
     pl->stat_part_cap = 2 * 2 * conv_blocks + 2 * (int64_t)ns * harm_blocks;
@@ -1236,7 +1240,6 @@ jerk_status jerk_search_range(jerk_plan pl, const void *d_spec, int64_t n, int32
     const float2 *in[1] = {(const float2 *)d_spec};
     s = enqueue_search(pl, in, st, false, false);
     if (s != JERK_OK) return s;
-    JCHECK(cudaMemsetAsync(pl->d_count, 0, sizeof(unsigned long long), st));   // no candidates yet
     s = finish_search(pl, st, 1, false);
     pl->partial = true;
     return s;
@@ -1289,6 +1292,7 @@ jerk_status jerk_select(jerk_plan pl, const double *h_sum, const double *h_sumsq
     JCHECK(cudaStreamWaitEvent(st, pl->done, 0));
     JCHECK(cudaMemcpyAsync(pl->d_stats, stats, sizeof(double) * 2 * ns, cudaMemcpyHostToDevice, st));
     JCHECK(cudaMemcpyAsync(pl->d_theta, theta, sizeof(float) * ns, cudaMemcpyHostToDevice, st));
+    JCHECK(cudaMemsetAsync(pl->d_count, 0, sizeof(unsigned long long), st));
     const jerk_status s = enqueue_peaks(pl, st);
     if (s != JERK_OK) return s;
     JCHECK(cudaStreamSynchronize(st));             // the host arrays above are on the stack
