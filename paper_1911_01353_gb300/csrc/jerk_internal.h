@@ -167,6 +167,17 @@ struct PeakArgs {
     unsigned long long *count;
 };
 
+// A search's results in the plan's pinned host memory, written by its last
+// kernel: the error flag, the candidate count, the first candidates, and per
+// item the statistics and thresholds.
+constexpr int kFirstCands = 1024;
+struct HostResult {
+    int err;
+    unsigned long long count;
+    DevCand cand[kFirstCands];
+    // then double stats[items][2 JERK_MAX_STAGES], float theta[items][JERK_MAX_STAGES]
+};
+
 // what a search clears before it starts: the max-projections' used parts and the candidate count
 struct ClearArgs {
     unsigned long long *M[JERK_MAX_STAGES];
@@ -208,6 +219,9 @@ cudaError_t launch_finalise_stats(const ItemDesc *items, int n_items, const doub
                                   int n_stages, const double *counts, const float *thresh, int mode,
                                   double *stats_out, float *theta_out, cudaStream_t st);
 cudaError_t launch_peaks(const PeakArgs &a, int n_items, int n_stages, int64_t most_cells, int sms, cudaStream_t st);
+cudaError_t launch_publish(HostResult *res, double *h_stats, float *h_theta, int n_items, const int *err,
+                           const unsigned long long *count, int64_t cap, const DevCand *cand, const double *stats,
+                           const float *theta, cudaStream_t st);
 cudaError_t launch_clear(const ClearArgs &a, int sms, cudaStream_t st);
 cudaError_t launch_wait_check(int *err, uint64_t limit_ns, cudaStream_t st);
 cudaError_t measure_peaks(int sms, double *fp32_tflops, double *l2_gbs);
@@ -329,5 +343,8 @@ struct jerk_plan_s {
     cudaEvent_t done = nullptr;
     bool profile = false, profiled = false;
     cudaEvent_t ev[JERK_N_PHASES + 1] = {};
-    jerk::DevCand *h_cand = nullptr;   // pinned staging for candidates
+    jerk::DevCand *h_cand = nullptr;   // pinned staging for candidates past the first kFirstCands
+    jerk::HostResult *h_res = nullptr; // pinned: what the last search's publish kernel wrote
+    double *h_stats = nullptr;         // in h_res' allocation, [max_batch][2 JERK_MAX_STAGES]
+    float *h_theta = nullptr;          // the same, [max_batch][JERK_MAX_STAGES]
 };

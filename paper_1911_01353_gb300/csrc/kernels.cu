@@ -612,6 +612,38 @@ cudaError_t launch_clear(const ClearArgs &a, int sms, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
+// The results into pinned host memory (one block; only what is there is
+// written), so that reading them costs the host one event wait: four blocking
+// copies for the candidates and three for each item's statistics took
+// 10 us each, more than the kernels of a 2^16-bin search.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) publish_kernel(HostResult *res, double *h_stats, float *h_theta, int n_items,
+                                                      const int *err, const unsigned long long *count, int64_t cap,
+                                                      const DevCand *cand, const double *stats, const float *theta) {
+    for (int i = threadIdx.x; i < n_items * 2 * JERK_MAX_STAGES; i += blockDim.x) h_stats[i] = stats[i];
+    for (int i = threadIdx.x; i < n_items * JERK_MAX_STAGES; i += blockDim.x) h_theta[i] = theta[i];
+    if (cand) {
+        const unsigned long long c = *count;
+        int64_t n = c < (unsigned long long)cap ? (int64_t)c : cap;
+        if (n > kFirstCands) n = kFirstCands;
+        constexpr int W = sizeof(DevCand) / 8;
+        const unsigned long long *src = reinterpret_cast<const unsigned long long *>(cand);
+        unsigned long long *dst = reinterpret_cast<unsigned long long *>(res->cand);
+        for (int64_t i = threadIdx.x; i < n * W; i += blockDim.x) dst[i] = src[i];
+        if (threadIdx.x == 0) res->count = c;
+    }
+    if (threadIdx.x == 0) res->err = *err;
+}
+
+cudaError_t launch_publish(HostResult *res, double *h_stats, float *h_theta, int n_items, const int *err,
+                           const unsigned long long *count, int64_t cap, const DevCand *cand, const double *stats,
+                           const float *theta, cudaStream_t st) {
+    static_assert(sizeof(DevCand) % 8 == 0, "copied as 8-byte words");
+    publish_kernel<<<1, 256, 0, st>>>(res, h_stats, h_theta, n_items, err, count, cap, cand, stats, theta);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
 // Failure-path check: one thread waits, with the filter kernels' bounded
 // wait, on a phase of an mbarrier that nothing completes; when the limit
 // expires it sets the device error flag exactly as a filter CTA would, and

@@ -311,6 +311,7 @@ void release(jerk_plan_s *pl) {
     cudaFree(pl->d_chk);
     cudaFree(pl->d_tc);
     if (pl->h_cand) cudaFreeHost(pl->h_cand);
+    if (pl->h_res) cudaFreeHost(pl->h_res);
     if (pl->done) cudaEventDestroy(pl->done);
     for (auto &e : pl->ev)
         if (e) cudaEventDestroy(e);
@@ -624,6 +625,12 @@ jerk_status transient_layout(jerk_plan_s *pl, const std::vector<int64_t> &n, con
 // host synchronisation, no event waits).
 jerk_status enqueue_peaks(jerk_plan_s *pl, cudaStream_t st);
 
+// the results of the current layout's search into the plan's pinned memory
+cudaError_t publish(jerk_plan_s *pl, cudaStream_t st) {
+    return launch_publish(pl->h_res, pl->h_stats, pl->h_theta, (int)pl->cur->n.size(), pl->d_err, pl->d_count,
+                          pl->prm.max_candidates, pl->d_cand, pl->d_stats, pl->d_theta, st);
+}
+
 jerk_status enqueue_search(jerk_plan_s *pl, const float2 *const *in, cudaStream_t st, bool capturing,
                            bool peaks = true) {
     const BatchLayout &L = *pl->cur;
@@ -704,6 +711,7 @@ jerk_status enqueue_search(jerk_plan_s *pl, const float2 *const *in, cudaStream_
         const jerk_status ps = enqueue_peaks(pl, st);     // (the count is cleared above)
         if (ps != JERK_OK) return ps;
     }
+    JCHECK(publish(pl, st));
     JCHECK(mark(pl, 5, st, capturing));
     return JERK_OK;
 }
@@ -723,14 +731,17 @@ jerk_status enqueue_peaks(jerk_plan_s *pl, cudaStream_t st) {
 }
 
 // after a synchronisation point: did a bounded device wait expire?
+jerk_status take_error(jerk_plan_s *pl, int err) {
+    if (!err) return JERK_OK;
+    cudaMemset(pl->d_err, 0, sizeof(int));
+    pl->h_res->err = 0;
+    return JERK_ETIMEOUT;
+}
+
 jerk_status device_error(jerk_plan_s *pl) {
     int err = 0;
     JCHECK(cudaMemcpy(&err, pl->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (err) {
-        cudaMemset(pl->d_err, 0, sizeof(int));
-        return JERK_ETIMEOUT;
-    }
-    return JERK_OK;
+    return take_error(pl, err);
 }
 
 jerk_status finish_search(jerk_plan_s *pl, cudaStream_t st, int count, bool profiled) {
@@ -930,6 +941,14 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
     TRY(dalloc(&pl->bytes, &pl->d_chk, 2));
     TRY(cudaMemset(pl->d_chk, 0, 2 * sizeof(long long)));
     TRY(cudaMallocHost((void **)&pl->h_cand, sizeof(DevCand) * (size_t)params->max_candidates));
+    TRY(cudaMallocHost((void **)&pl->h_res, sizeof(HostResult) + (size_t)pl->max_batch * JERK_MAX_STAGES *
+                                                                    (2 * sizeof(double) + sizeof(float))));
+    if (e == cudaSuccess) {
+        pl->h_res->err = 0;
+        pl->h_res->count = 0;
+        pl->h_stats = (double *)(pl->h_res + 1);
+        pl->h_theta = (float *)(pl->h_stats + (size_t)2 * JERK_MAX_STAGES * pl->max_batch);
+    }
     TRY(cudaEventCreateWithFlags(&pl->done, cudaEventDisableTiming));
     TRY(cudaMemcpy(pl->d_thresh, params->thresh, sizeof(float) * JERK_MAX_STAGES, cudaMemcpyHostToDevice));
 #undef TRY
@@ -1208,6 +1227,9 @@ jerk_status jerk_plane(jerk_plan pl, const void *d_spec, int64_t n, int32_t t0, 
     const int n_ctas = (int)(last - first);
     JCHECK(pl->prm.precision ? launch_conv_tc(pl->prm.precision, 1, false, a, n_ctas, st)
                              : launch_conv(pl->log2L, 1, false, a, n_ctas, st));
+    // an expired wait of this call is reported by the next read of results, as a search's is
+    JCHECK(launch_publish(pl->h_res, pl->h_stats, pl->h_theta, 0, pl->d_err, pl->d_count, 0, nullptr, pl->d_stats,
+                          pl->d_theta, st));
     JCHECK(cudaEventRecord(pl->done, st));
     return JERK_OK;
 }
@@ -1295,6 +1317,7 @@ jerk_status jerk_select(jerk_plan pl, const double *h_sum, const double *h_sumsq
     JCHECK(cudaMemsetAsync(pl->d_count, 0, sizeof(unsigned long long), st));
     const jerk_status s = enqueue_peaks(pl, st);
     if (s != JERK_OK) return s;
+    JCHECK(publish(pl, st));
     JCHECK(cudaStreamSynchronize(st));             // the host arrays above are on the stack
     JCHECK(cudaEventRecord(pl->done, st));
     pl->partial = false;
@@ -1395,16 +1418,19 @@ jerk_status jerk_candidates(jerk_plan pl, jerk_candidate *h_out, int64_t cap, in
     if (!pl->searched || pl->partial) return JERK_ESTATE;
     JCHECK(cudaSetDevice(pl->device));
     JCHECK(cudaEventSynchronize(pl->done));
-    {
-        const jerk_status de = device_error(pl);
-        if (de != JERK_OK) return de;
-    }
-    unsigned long long cnt = 0;
-    JCHECK(cudaMemcpy(&cnt, pl->d_count, sizeof(cnt), cudaMemcpyDeviceToHost));
+    const jerk_status de = take_error(pl, pl->h_res->err);
+    if (de != JERK_OK) return de;
+    const unsigned long long cnt = pl->h_res->count;
     const int64_t kept = std::min<int64_t>((int64_t)cnt, pl->prm.max_candidates);
-    if (kept > 0)
+    *n_out = (int64_t)cnt;
+    const jerk_status over = (int64_t)cnt > pl->prm.max_candidates || (int64_t)cnt > cap ? JERK_EOVERFLOW : JERK_OK;
+    if (cap == 0) return over;
+    const DevCand *from = pl->h_res->cand;
+    if (kept > kFirstCands) {
         JCHECK(cudaMemcpy(pl->h_cand, pl->d_cand, sizeof(DevCand) * (size_t)kept, cudaMemcpyDeviceToHost));
-    std::vector<DevCand> v(pl->h_cand, pl->h_cand + kept);
+        from = pl->h_cand;
+    }
+    std::vector<DevCand> v(from, from + kept);
     std::sort(v.begin(), v.end(), [](const DevCand &x, const DevCand &y) {
         if (x.item != y.item) return x.item < y.item;
         return x.stage_idx != y.stage_idx ? x.stage_idx < y.stage_idx : x.p < y.p;
@@ -1425,9 +1451,7 @@ jerk_status jerk_candidates(jerk_plan pl, jerk_candidate *h_out, int64_t cap, in
         c.power = d.power;
         c.item = d.item;
     }
-    *n_out = (int64_t)cnt;
-    if ((int64_t)cnt > pl->prm.max_candidates || (int64_t)cnt > cap) return JERK_EOVERFLOW;
-    return JERK_OK;
+    return over;
 }
 
 jerk_status jerk_maxproj(jerk_plan pl, int32_t item, int32_t stage_idx, const uint64_t **d_out,
@@ -1524,14 +1548,10 @@ jerk_status jerk_stats(jerk_plan pl, int32_t item, double *h_mean, double *h_std
     if (item < 0 || item >= pl->last_count) return JERK_EINVAL;
     JCHECK(cudaSetDevice(pl->device));
     JCHECK(cudaEventSynchronize(pl->done));
-    {
-        const jerk_status de = device_error(pl);
-        if (de != JERK_OK) return de;
-    }
-    double st[2 * JERK_MAX_STAGES];
-    float th[JERK_MAX_STAGES];
-    JCHECK(cudaMemcpy(st, pl->d_stats + (size_t)item * 2 * JERK_MAX_STAGES, sizeof(st), cudaMemcpyDeviceToHost));
-    JCHECK(cudaMemcpy(th, pl->d_theta + (size_t)item * JERK_MAX_STAGES, sizeof(th), cudaMemcpyDeviceToHost));
+    const jerk_status de = take_error(pl, pl->h_res->err);
+    if (de != JERK_OK) return de;
+    const double *st = pl->h_stats + (size_t)item * 2 * JERK_MAX_STAGES;
+    const float *th = pl->h_theta + (size_t)item * JERK_MAX_STAGES;
     for (int si = 0; si < pl->prm.n_stages; ++si) {
         if (h_mean) h_mean[si] = st[2 * si];
         if (h_std) h_std[si] = st[2 * si + 1];
