@@ -11,19 +11,40 @@ namespace jerk {
 // bins, med = element of rank floor((n-1)/2) of |F_k|^2 (FP64, exact for
 // FP32 input), F_k <- F_k (med / ln 2)^(-1/2).
 //
-// One warp per block of up to 1024 bins (four warps above), every bin's power
-// rounded to FP32 in a register: rounding keeps the order, so bisecting the
-// FP32 bit patterns by counting (one compare per bin and step, one warp
-// reduction, no barrier) closes in on the powers around the median, and the
-// FP64 powers decide among those that are left, one as a rule after 15 to 20
-// steps.  What bounds it is the FP64 pipe (8 operations and conversions per
-// bin); the bitonic sort of all FP64 powers that this replaces spent 55
-// barriers per block: 2^21 bins 170 -> 89 us, a batch of 24 spectra of 2^13-2^16
-// bins 555 -> 40 us (one launch normalises up to kNormItems spectra).
+// Each block's powers are formed in FP32 (at most 2^-22 off, relatively) and
+// kept in registers; bisecting their bit patterns by counting (one compare per
+// bin and step, one warp reduction) closes in on the FP32 median v.  The FP64
+// median then lies within a few units in the last place of v: the FP64 powers
+// of the bins that close decide, one or two bins as a rule.  Bins are scaled by
+// the FP64 factor as a pair of floats, with the FP64 product where the pair
+// cannot decide the rounding, so that the result is the FP64 one bit for bit.
+// FP64 instructions run at 1/64 of the FP32 rate, and sorting all FP64 powers
+// (55 barriers), then keying and scaling all bins in FP64, were the longest
+// parts: 2^16 bins 24 -> 9 us, 2^21 bins 170 -> 89 -> 76 us, a batch of 24
+// spectra of 2^13-2^16 bins 555 -> 40 -> 34 us.  Blocks that are too small or too large for FP32
+// powers take the FP64 powers rounded to FP32, which keep the order.  One warp
+// per block of up to 1024 bins (four above, or where there are few blocks);
+// one launch normalises up to kNormItems spectra.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned long long power_key(float2 f) {
     const double re = f.x, im = f.y;
     return (unsigned long long)__double_as_longlong(re * re + im * im);   // non-negative: integer order = value order
+}
+
+// (float)((double)f * scale), scale = sh + sl to 2^-48.  The product as a pair
+// p + e is good to 2^-46 of it; it decides the rounding unless what is left
+// after rounding lies within 2^-18 of half a unit in the last place, the result
+// is a power of two (the unit changes there) or out of the normal range.
+__device__ __forceinline__ float scaled(float f, double scale, float sh, float sl) {
+    const float p = __fmul_rn(f, sh);
+    const float e = __fmaf_rn(f, sl, __fmaf_rn(f, sh, -p));
+    const float r = __fadd_rn(p, e);
+    const float left = fabsf(__fadd_rn(__fsub_rn(p, r), e));
+    const unsigned bits = __float_as_uint(r);
+    const float half = __uint_as_float(bits & 0x7f800000u) * 5.9604644775390625e-8f;   // 2^-24 of r's power of two
+    const float a = fabsf(r);
+    if (fabsf(left - half) > half * 3.8e-6f && (bits & 0x007fffffu) != 0u && a >= 1e-28f && a <= 1e28f) return r;
+    return (float)((double)f * scale);
 }
 
 // sums and extrema over the W warps of a block of bins
@@ -75,38 +96,73 @@ __global__ void __launch_bounds__(32 * W) normalise_kernel(NormArgs a, int B) {
     const float2 *in = a.in[item] + s0;
     float2 *out = a.out[item] + s0;
     const int tid = threadIdx.x;
+    // FP32 powers, or FP64 ones rounded to FP32 (exact: both keep the order of the FP64 powers)
     unsigned key[KPT];
-    unsigned lo = ~0u, hi = 0u;
-#pragma unroll
-    for (int i = 0; i < KPT; ++i) {
-        const int k = tid + NT * i;
-        key[i] = ~0u;                                         // above every power: never counted
-        if (k < nb) {
-            key[i] = __float_as_uint((float)__longlong_as_double((long long)power_key(in[k])));
-            lo = min(lo, key[i]);
-            hi = max(hi, key[i]);
-        }
-    }
-    lo = BlockOf<W>::low(lo);
-    hi = BlockOf<W>::high(hi);
-    // the median is one of the n_hi - n_lo powers in [lo, hi]
     const unsigned rank = (unsigned)(nb - 1) / 2;
-    unsigned n_lo = 0, n_hi = (unsigned)nb;
-    while (lo < hi && n_hi - n_lo > 1) {
-        const unsigned mid = lo + (hi - lo) / 2;
-        unsigned c = 0;
+    unsigned lo, hi, n_lo;
+    auto bisect = [&](bool exact) {
+        lo = ~0u;
+        hi = 0u;
 #pragma unroll
-        for (int i = 0; i < KPT; ++i) c += key[i] <= mid ? 1u : 0u;
-        c = BlockOf<W>::add(c);
-        if (c > rank) {
-            hi = mid;
-            n_hi = c;
+        for (int i = 0; i < KPT; ++i) {
+            const int k = tid + NT * i;
+            key[i] = ~0u;                                     // above every power: never counted
+            if (k < nb) {
+                const float2 f = in[k];
+                key[i] = exact ? __float_as_uint((float)__longlong_as_double((long long)power_key(f)))
+                               : __float_as_uint(fmaf(f.x, f.x, f.y * f.y));
+                lo = min(lo, key[i]);
+                hi = max(hi, key[i]);
+            }
+        }
+        lo = BlockOf<W>::low(lo);
+        hi = BlockOf<W>::high(hi);
+        // the key of that rank is one of the n_hi - n_lo in [lo, hi]
+        unsigned n_hi = (unsigned)nb;
+        n_lo = 0;
+        while (lo < hi && n_hi - n_lo > 1) {
+            const unsigned mid = lo + (hi - lo) / 2;
+            unsigned c0 = 0, c1 = 0, c2 = 0, c3 = 0;          // four counts: short chains
+#pragma unroll
+            for (int i = 0; i < KPT; i += 4) {
+                c0 += key[i] <= mid ? 1u : 0u;
+                c1 += key[i + 1] <= mid ? 1u : 0u;
+                c2 += key[i + 2] <= mid ? 1u : 0u;
+                c3 += key[i + 3] <= mid ? 1u : 0u;
+            }
+            const unsigned c = BlockOf<W>::add((c0 + c1) + (c2 + c3));
+            if (c > rank) {
+                hi = mid;
+                n_hi = c;
+            } else {
+                lo = mid + 1;
+                n_lo = c;
+            }
+        }
+    };
+    bisect(false);
+    {
+        // narrow [lo, hi] to the one key of that rank: the smallest in it at or above lo
+        unsigned v = ~0u;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+            if (key[i] >= lo && key[i] <= hi) v = min(v, key[i]);
+        v = BlockOf<W>::low(v);
+        const float fv = __uint_as_float(v);
+        if (fv >= 1e-30f && fv <= 1e30f) {
+            // |FP32 power - FP64 power| <= 2^-22 of it, so is the median's distance from v: a bin
+            // 8 units in the last place (2^-21 or more of v) below v is below the median
+            lo = v - 8;
+            hi = v + 8;
+            unsigned c = 0;
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) c += key[i] < lo ? 1u : 0u;
+            n_lo = BlockOf<W>::add(c);
         } else {
-            lo = mid + 1;
-            n_lo = c;
+            bisect(true);
         }
     }
-    // among them, by FP64 powers: their range, then by counting again if it is wider than one value
+    // among the bins in [lo, hi], by FP64 powers: their range, then by counting again if it is wider than one value
     unsigned long long lo64 = ~0ull, hi64 = 0ull;
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
@@ -132,18 +188,20 @@ __global__ void __launch_bounds__(32 * W) normalise_kernel(NormArgs a, int B) {
     }
     const double med = __longlong_as_double((long long)lo64);
     const double scale = med > 0.0 ? 1.0 / sqrt(med / 0.69314718055994530942) : 1.0;
+    const float sh = (float)scale, sl = (float)(scale - (double)sh);
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
         const int k = tid + NT * i;
         if (k < nb) {
             const float2 f = in[k];
-            out[k] = make_float2((float)((double)f.x * scale), (float)((double)f.y * scale));
+            out[k] = make_float2(scaled(f.x, scale, sh, sl), scaled(f.y, scale, sh, sl));
         }
     }
 }
 
 cudaError_t launch_normalise(const float2 *const *in, float2 *const *out, const int64_t *n, int count, int B,
                              cudaStream_t st) {
+    const int64_t sms = current_device_sms();
     for (int i0 = 0; i0 < count; i0 += kNormItems) {
         NormArgs a;
         a.count = count - i0 < kNormItems ? count - i0 : kNormItems;
@@ -158,6 +216,8 @@ cudaError_t launch_normalise(const float2 *const *in, float2 *const *out, const 
         if (blk > INT32_MAX) return cudaErrorInvalidValue;
         if (B <= 256)
             normalise_kernel<8, 1><<<(unsigned)blk, 32, 0, st>>>(a, B);
+        else if (B <= 1024 && blk <= sms)
+            normalise_kernel<8, 4><<<(unsigned)blk, 128, 0, st>>>(a, B);
         else if (B <= 1024)
             normalise_kernel<32, 1><<<(unsigned)blk, 32, 0, st>>>(a, B);
         else

@@ -24,6 +24,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kTable = 1024;         // templates whose harmonic indices are in shared memory at a time
+constexpr int kAhead = 4;            // templates whose loads are in flight together
 constexpr int kFlush = 32;           // sums between two additions to the FP64 statistics
 
 // a h / H to the nearest integer, halves away from zero
@@ -70,6 +71,13 @@ __global__ void __launch_bounds__(kThreads) subharmonic_kernel(SubArgs a) {
     __shared__ double r1[kWarps], r2[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double s1 = 0.0, s2 = 0.0;
+    PairSum p1, p2;
+    int k = 0;                               // sums in p1, p2
+    auto flush = [&] {
+        p1.flush(s1);
+        p2.flush(s2);
+        k = 0;
+    };
     for (int64_t q0 = 32 * (int64_t)blockIdx.x; q0 < a.bN; q0 += 32 * (int64_t)gridDim.x) {
         const int64_t q = q0 + lane;
         const bool in = q < a.bN;
@@ -90,45 +98,52 @@ __global__ void __launch_bounds__(kThreads) subharmonic_kernel(SubArgs a) {
                 }
                 __syncthreads();
             }
-            // this warp's part, ascending; parts and tables ascend too
+            // this warp's part, ascending; parts and tables ascend too.  kAhead
+            // templates at a time, their loads issued before the first is used
             const int i1 = (int)((int64_t)n * (warp + 1) / kWarps);
-            PairSum p1, p2;
-            int k = 0;
             float pb = -1.0f;
             int pt = 0;
-#pragma unroll 4
-            for (int i = (int)((int64_t)n * warp / kWarps); i < i1; ++i) {
-                float S = 0.0f;
+            for (int i = (int)((int64_t)n * warp / kWarps); i < i1; i += kAhead) {
+                float S[kAhead];
+                const int u1 = min(kAhead, i1 - i);
 #pragma unroll
-                for (int h = 0; h < H; ++h) S += __ldg(col[h] + (int64_t)row[i][h] * a.bN);
-                if (S > pb) {
-                    pb = S;
-                    pt = tb + i;
+                for (int u = 0; u < kAhead; ++u) {
+                    const int e = i + min(u, u1 - 1);
+                    S[u] = 0.0f;
+#pragma unroll
+                    for (int h = 0; h < H; ++h) S[u] += __ldg(col[h] + (int64_t)row[e][h] * a.bN);
+                }
+                float top = S[0], low = S[0];
+                bool nan = false;
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    if (u < u1 && S[u] > pb) {
+                        pb = S[u];
+                        pt = tb + i + u;
+                    }
+                    top = fmaxf(top, S[u]);
+                    low = fminf(low, S[u]);
+                    nan = nan || !(S[u] == S[u]);
                 }
                 // S and S^2 as exact pairs in the range where both are normal numbers, else in FP64
-                if (S == 0.0f || (S >= 1e-12f && S <= 1e15f)) {
-                    p1.add(S);
-                    const float sq = __fmul_rn(S, S);
-                    p2.add(sq);
-                    p2.c = __fadd_rn(p2.c, __fmaf_rn(S, S, -sq));
+                if (low >= 1e-12f && top <= 1e15f && !nan) {
+#pragma unroll
+                    for (int u = 0; u < kAhead; ++u) {
+                        const float x = u < u1 && in ? S[u] : 0.f;
+                        const float sq = __fmul_rn(x, x);
+                        p1.add(x);
+                        p2.add(sq);
+                        p2.c = __fadd_rn(p2.c, __fmaf_rn(x, x, -sq));
+                    }
+                    k += kAhead;
                 } else if (in) {
-                    s1 += (double)S;
-                    s2 += (double)S * (double)S;
-                }
-                if (++k == kFlush) {
-                    k = 0;
-                    if (in) {
-                        p1.flush(s1);
-                        p2.flush(s2);
-                    } else {
-                        p1 = PairSum();
-                        p2 = PairSum();
+                    for (int u = 0; u < u1; ++u) {
+                        const double x = u == 0 ? S[0] : u == 1 ? S[1] : u == 2 ? S[2] : S[3];
+                        s1 += x;
+                        s2 += x * x;
                     }
                 }
-            }
-            if (in) {
-                p1.flush(s1);
-                p2.flush(s2);
+                if (k >= kFlush) flush();
             }
             smax[warp][lane] = pb;
             sarg[warp][lane] = pt;
@@ -147,6 +162,7 @@ __global__ void __launch_bounds__(kThreads) subharmonic_kernel(SubArgs a) {
             a.M[q] = ((unsigned long long)__float_as_uint(best) << 32) |
                      (unsigned long long)(0xFFFFFFFFu - (unsigned)bt);
     }
+    flush();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         s1 += __shfl_xor_sync(0xffffffffu, s1, o);
