@@ -14,9 +14,22 @@
 //   twiddle U'[k1][n2] = D1 w^{k1 n2}   (FP32, in registers)
 //   step 3: D3 = A3 B      A3[(seg, n2)][(re/im, k1)] = U'         (MN-major)
 // where B is the real block form of F (the same matrix for both steps, F is
-// symmetric).  D1 and D3 sit in tensor memory; every thread reads one row
-// (tcgen05.ld), so the power |y|^2, the running max over the template group,
-// the statistics and the harmonic rows are computed as in the FP32 kernel.
+// symmetric).  D1 and then D3 sit in the same 128 columns of tensor memory;
+// every thread reads half of one row (tcgen05.ld), so the power |y|^2, the
+// running max over the template group, the statistics and the harmonic rows are
+// computed as in the FP32 kernel.
+//
+// Two groups of eight warps share the two segments and take the templates in
+// turn, each with a template buffer, an operand and an accumulator of its own.
+// Within a group the phases follow one another (operand build, step 1, twiddle,
+// step 3, power); the other group fills the waits on products, tensor memory
+// and barriers.  With all 16 warps on one template, barriers of the whole CTA
+// kept them in the same phase and 42 % of the issue slots busy.  The segment
+// spectra sit in tensor memory too (64 columns per thread), which makes room in
+// registers for the 32 running maxima a thread has in this layout.  Bank of
+// 12 261 templates, 2^20 bins, FP16: filter 50.3 -> 44.7 ms, results unchanged
+// bit for bit.  The bound is still latency: shared memory (operands, template,
+// twiddles and the products' own reads) 55 %, issue 43 %, tensor pipe 31 %.
 //
 // Scaling: each segment spectrum is divided by max|X| * max|C| over the bank,
 // so |Z| <= 1 and the FP16 operands of both steps stay in range (|U'| <= 64,
@@ -36,6 +49,7 @@
 #include "device_sync.cuh"
 #include "fft.cuh"
 #include "jerk_internal.h"
+#include "tmem.cuh"
 
 namespace jerk {
 namespace {
@@ -45,14 +59,15 @@ constexpr int WPAD = L + L / 16;                          // forward-transform w
 constexpr uint32_t LBO = 128;                             // operand core-matrix stride along K (bytes)
 constexpr uint32_t SBO = 2048;                            // ... along M / N (16 cores of 128 B along K)
 constexpr int OPB = 128 * 128 * 2;                        // one 16-bit 128 x 128 operand
-constexpr int OFF_A1 = 2 * L * 8;                         // after the two-deep template ring
-constexpr int OFF_A3 = OFF_A1 + OPB;
-constexpr int OFF_B = OFF_A3 + OPB;                       // B, then the twiddle table (one bulk copy)
+constexpr int GT = THREADS / 2;                           // threads of a group (one template at a time)
+constexpr int kFlush = 256;                               // templates of a group per 8-bit argmax
+constexpr int OFF_A = 2 * L * 8;                          // after the groups' template buffers: one operand each
+constexpr int OFF_B = OFF_A + 2 * OPB;                    // B, then the twiddle table (one bulk copy)
 constexpr int OFF_TW = OFF_B + OPB;                       // w^{k1 n2} for n2 = 2p, 2p + 1: float4 [p][k1] (re, re, im, im)
-constexpr int OFF_AMX = OFF_TW + 64 * 64 * 8;             // uint16 [SEGS][L]: argmax offset in the group
-constexpr int SMEM = OFF_AMX + SEGS * L * 2;              // 212 992 bytes
-constexpr uint32_t TMEM_COLS = 256;                       // D1: columns 0..127, D3: 128..255
-static_assert(SEGS * WPAD * 8 <= OFF_A3, "forward-transform work must fit below A3");
+constexpr int OFF_AMX = OFF_TW + 64 * 64 * 8;             // uint8 [2][32][GT]: argmax among a group's last kFlush
+constexpr int SMEM = OFF_AMX + 2 * 32 * GT;               // 212 992 bytes
+constexpr uint32_t TMEM_COLS = 512;                       // a group's D: 128 g ..; spectrum values: 256 + 64 (warp / 4) ..
+static_assert(SEGS * WPAD * 8 <= OFF_B, "forward-transform work must fit below B");
 
 template <int PREC>
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
@@ -128,12 +143,13 @@ __device__ __forceinline__ void mma_commit_warp(uint64_t *bar) {
         : "memory");
 }
 
-// st.shared.u16 under a predicate, with no branch around it
-__device__ __forceinline__ void st_shared_u16_if(bool pred, uint32_t addr, uint16_t v) {
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q st.shared.u16 [%1], %2;\n\t}" ::"r"((uint32_t)pred),
-        "r"(addr), "h"(v)
-        : "memory");
+// mx = max(mx, p), and v's low byte to shared memory where p is the larger: a
+// compare, a predicated store and a maximum, with no branch (rare after the
+// first templates)
+__device__ __forceinline__ void max_arg(float p, float &mx, uint32_t addr, int v) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.gt.f32 q, %0, %1;\n\t@q st.shared.u8 [%2], %3;\n\t}" ::"f"(p), "f"(mx),
+                 "r"(addr), "r"(v));
+    mx = fmaxf(mx, p);
 }
 
 // acc0 += x0, acc1 += x1 in FP64.  A call, not inlined, so that it stays
@@ -189,24 +205,25 @@ __device__ __forceinline__ int tc_bank_row(const ConvArgs &a, int k) {
 template <int PREC, int MODE, bool STATS, bool ROWS>
 __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
     extern __shared__ __align__(1024) unsigned char sm[];
-    float2 *ring = reinterpret_cast<float2 *>(sm);
-    uint16_t *amx_s = reinterpret_cast<uint16_t *>(sm + OFF_AMX);
-    __shared__ __align__(8) uint64_t full[2];                 // template bulk copy landed
-    __shared__ __align__(8) uint64_t mbar1, mbar3, cbar;      // step 1 / step 3 done; constants landed
+    __shared__ __align__(8) uint64_t full[2];                 // a group's template landed
+    __shared__ __align__(8) uint64_t mbar1[2], mbar3[2], cbar; // a group's step 1 / step 3 done; constants landed
     __shared__ int issued[2];
     __shared__ uint32_t tmem_slot;
     __shared__ int xmax_bits[SEGS];
     __shared__ double red[2][THREADS / 32];
     __shared__ double dacc[STATS ? 2 : 1][STATS ? THREADS : 1];
-    __shared__ __align__(16) TplMeta tq[4];                 // (t, e0, e1) of template k at [k & 3]
-    __shared__ __align__(16) RowEntries rent[2];            // slot entries of template k at [k & 1]
+    __shared__ __align__(16) TplMeta tq[2][4];                // (t, e0, e1) of a group's template i at [i & 3]
+    __shared__ __align__(16) RowEntries rent[2][2];           // its slot entries at [i & 1]
 
     const int tid = threadIdx.x;
     const int half = tid / NT, j = tid % NT;                  // forward-transform mapping
     const int warp = tid >> 5, lane = tid & 31;
-    const int quarter = warp & 3, gcol = warp >> 2;           // tensor-memory lane quarter, column group
+    const int grp = tid / GT, gt = tid % GT, gwarp = gt >> 5; // group and place in it
+    const int quarter = gwarp & 3, gcol = gwarp >> 2;         // tensor-memory lane quarter, column half
     const int row = 32 * quarter + lane;                      // operand / accumulator row: (seg, r)
     const int seg = row >> 6, r = row & 63;
+    float2 *buf = reinterpret_cast<float2 *>(sm) + grp * L;   // this group's template
+    unsigned char *opa = sm + OFF_A + grp * OPB;              // its operand A (step 1's, then step 3's)
 
     // (spectrum, template group) entry of this CTA
     const int cta = (int)blockIdx.x + a.cta_base;
@@ -223,22 +240,20 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
     }
     const int s_base = (cta - __ldg(&a.grp[lo].cta0)) * SEGS;
     const int64_t bN = itm->bN;
+    const int nt = te - tb;                                   // templates of the CTA; group g takes g, g + 2, ..
+    const int ng = (nt - grp + 1) >> 1;                       // this group's templates
 
     if (tid == 0) {
-        mbar_init(&full[0], 1);
-        mbar_init(&full[1], 1);
-        mbar_init(&mbar1, 1);
-        mbar_init(&mbar3, 1);
+        for (int g = 0; g < 2; ++g) {
+            mbar_init(&full[g], 1);
+            mbar_init(&mbar1[g], 1);
+            mbar_init(&mbar3[g], 1);
+            issued[g] = 0;
+        }
         mbar_init(&cbar, 1);
-        issued[0] = issued[1] = 0;
         xmax_bits[0] = xmax_bits[1] = 0;
     }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                     "r"(TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (warp == 0) tmem_alloc_warp(smem_u32(&tmem_slot), TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -273,25 +288,23 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
         for (int m = 0; m < 16; ++m) work[rv + NT * m] = v[m];   // natural order
     }
     __syncthreads();
-    // this thread's spectrum values in the tensor-core mapping: X[seg][r + 64 (16 gcol + i)]
-    // Operand-build mapping: thread (ka, blk) forms Z for k = ka + 64 k2, k2 in
-    // [8 blk, 8 blk + 8), of BOTH segments, so each template value is read from
-    // shared memory once per CTA.  It keeps X[s][ka + 64 (8 blk + i)], s = 0, 1.
-    // Values i and i + 1 are kept as packed pairs (xr: real parts, xi:
-    // imaginary parts), matching the bank's paired form (f, f + 64).
-    const int ka = tid & 63, blk = tid >> 6;
-    float2 xr[SEGS][4], xi[SEGS][4];
+    // Operand-build mapping: thread (ka, blk) of each group forms Z for k = ka + 64 k2,
+    // k2 in [16 blk, 16 blk + 16), of BOTH segments, so each template value is read
+    // from shared memory once.  Its spectrum values X[s][ka + 64 (16 blk + i)] sit
+    // in its tensor-memory columns, values i and i + 1 as packed pairs matching
+    // the bank's paired form: column 32 c + 16 s + 4 p: (re, re, im, im) of i =
+    // 8 c + 2 p, + 1.
+    const int ka = gt & 63, blk = gt >> 6;
+    const uint32_t tx = tmem + tlane + 256 + 64 * (uint32_t)(warp >> 2);
     {
         float m[SEGS] = {0.f, 0.f};
 #pragma unroll
         for (int s2 = 0; s2 < SEGS; ++s2) {
-            const float2 *ws = reinterpret_cast<const float2 *>(sm) + s2 * WPAD;
+            const float2 *ws = reinterpret_cast<const float2 *>(sm) + s2 * WPAD + ka + 64 * 16 * blk;
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) {
-                const float2 x0 = ws[ka + 64 * (8 * blk + i)], x1 = ws[ka + 64 * (8 * blk + i + 1)];
-                xr[s2][i >> 1] = make_float2(x0.x, x1.x);
-                xi[s2][i >> 1] = make_float2(x0.y, x1.y);
-                m[s2] = fmaxf(m[s2], fmaxf(fmaxf(fabsf(x0.x), fabsf(x0.y)), fmaxf(fabsf(x1.x), fabsf(x1.y))));
+            for (int i = 0; i < 16; ++i) {
+                const float2 x = ws[64 * i];
+                m[s2] = fmaxf(m[s2], fmaxf(fabsf(x.x), fabsf(x.y)));
             }
         }
 #pragma unroll
@@ -301,32 +314,25 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
             if (lane == 0) atomicMax(&xmax_bits[s2], __float_as_int(m[s2]));   // non-negative: int order = float order
         }
     }
-    if (tid == 64 && tb < te) {
-        // the metadata pipeline's first stages: (t, e0, e1) of the first two
-        // templates, t of the third, the slot entries of the first (later ones
-        // are prefetched by cp.async in the loop)
-        // (plane mode needs t only: it has no slot tables)
-        for (int q = 0; q < 3 && tb + q < te; ++q) {
-            const int t = __ldg(a.order + tb + q);
+    if (gt == 64 && ng > 0) {
+        // the metadata pipeline's first stages: (t, e0, e1) of the group's first two
+        // templates, t of the third, the slot entries of the first (later ones are
+        // prefetched by cp.async in the loop; plane mode needs t only)
+        for (int q = 0; q < 3 && q < ng; ++q) {
+            const int t = __ldg(a.order + tb + 2 * q + grp);
             const bool ent = MODE == 0 && q < 2;
-            tq[(tb + q) & 3] = TplMeta{t, ent ? __ldg(a.slot_beg + t) : 0, ent ? __ldg(a.slot_beg + t + 1) : 0, 0};
+            tq[grp][q] = TplMeta{t, ent ? __ldg(a.slot_beg + t) : 0, ent ? __ldg(a.slot_beg + t + 1) : 0, 0};
         }
         if constexpr (MODE == 0) {
-            const TplMeta m0 = tq[tb & 3];
+            const TplMeta m0 = tq[grp][0];
             for (int i = 0; i < m0.e1 - m0.e0; ++i) {
-                rent[tb & 1].h[i] = __ldg(a.slot_h + m0.e0 + i);
-                rent[tb & 1].off[i] = __ldg(itm->slot_off + m0.e0 + i);
-                rent[tb & 1].len[i] = __ldg(itm->slot_len + m0.e0 + i);
+                rent[grp][0].h[i] = __ldg(a.slot_h + m0.e0 + i);
+                rent[grp][0].off[i] = __ldg(itm->slot_off + m0.e0 + i);
+                rent[grp][0].len[i] = __ldg(itm->slot_len + m0.e0 + i);
             }
         }
     }
-    __syncthreads();                                          // the work buffers are free from here
-    if (tid == 0)
-        for (int b = 0; b < 2 && tb + b < te; ++b) {
-            issued[b] = 1;
-            bulk_load(ring + b * L, a.bank + (int64_t)tc_bank_row<ROWS>(a, tb + b) * L, (uint32_t)(L * sizeof(float2)),
-                      &full[b]);
-        }
+    __syncthreads();
     float psc;                                                // power = |y|^2 * psc (segment seg)
     {
         const float cm = __ldg(a.tc_cmax);
@@ -334,279 +340,338 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
         for (int s2 = 0; s2 < SEGS; ++s2) {
             const float xm = __int_as_float(xmax_bits[s2]);
             const float sc = (xm > 0.f && cm > 0.f) ? 1.0f / (xm * cm) : 1.0f;
+            const float2 *ws = reinterpret_cast<const float2 *>(sm) + s2 * WPAD + ka + 64 * 16 * blk;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                xr[s2][i] = make_float2(xr[s2][i].x * sc, xr[s2][i].y * sc);
-                xi[s2][i] = make_float2(xi[s2][i].x * sc, xi[s2][i].y * sc);
-            }
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int p = 0; p < 4; p += 2) {
+                    float x[8];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const float2 x0 = ws[64 * (8 * c + 2 * (p + u))], x1 = ws[64 * (8 * c + 2 * (p + u) + 1)];
+                        x[4 * u] = x0.x * sc;
+                        x[4 * u + 1] = x1.x * sc;
+                        x[4 * u + 2] = x0.y * sc;
+                        x[4 * u + 3] = x1.y * sc;
+                    }
+                    tmem_st8(tx + 32 * c + 16 * s2 + 4 * p, x);
+                }
             if (s2 == seg) psc = 1.0f / (sc * sc);
         }
+        tmem_wait_st();
+    }
+    __syncthreads();                                          // the work buffers are free from here
+    if (gt == 0 && ng > 0) {
+        issued[grp] = 1;
+        bulk_load(buf, a.bank + (int64_t)tc_bank_row<ROWS>(a, tb + grp) * L, (uint32_t)(L * sizeof(float2)),
+                  &full[grp]);
     }
 
-    // cells of this thread: n = 64 (16 gcol + i) + r of segment seg.  n grows
-    // with i, so the valid ones (n < V and within the spectrum) are the first
-    // nvalid.
+    // cells of this thread: n = 64 (32 gcol + i) + r of segment seg, i < 32.  n
+    // grows with i, so the valid ones (n < V and within the spectrum) are the
+    // first nvalid.
     const int seg0 = (s_base + seg) * V;
     int nvalid = 0;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const int n = 64 * (16 * gcol + i) + r;
+    for (int i = 0; i < 32; ++i) {
+        const int n = 64 * (32 * gcol + i) + r;
         nvalid += (n < V && seg0 + n < bN) ? 1 : 0;
     }
-    float mx[16];
+    float mx[32];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) mx[i] = -1.0f;
+    for (int i = 0; i < 32; ++i) mx[i] = -1.0f;
     if constexpr (STATS) {
         dacc[0][tid] = 0.0;
         dacc[1][tid] = 0.0;
     }
     float c1 = 0.f, c2 = 0.f;
-    // A1 rows 64 s + ka, K chunk blk (re) and 8 + blk (im)
-    const uint32_t a1_r0 = smem_u32(sm + OFF_A1) + (ka >> 3) * SBO + (ka & 7) * 16 + blk * LBO;
+    // operand rows 64 s + ka, K chunks 2 blk, 2 blk + 1 (re) and 8 more (im)
+    const uint32_t a1_r0 = smem_u32(opa) + (ka >> 3) * SBO + (ka & 7) * 16 + 2 * blk * LBO;
     const uint32_t a1_r1 = a1_r0 + 8 * SBO;
-    const uint32_t a3_col = smem_u32(sm + OFF_A3) + (r >> 3) * LBO + (r & 7) * 16 + (8 * seg + 2 * gcol) * SBO;
-    const float4 *twt = reinterpret_cast<const float4 *>(sm + OFF_TW) + 8 * 64 * gcol + r;
-    const uint32_t amx_t = smem_u32(amx_s + seg * L + 64 * 16 * gcol + r);   // this thread's cells, stride 128 B
+    const uint32_t a3_col = smem_u32(opa) + (r >> 3) * LBO + (r & 7) * 16 + (8 * seg + 4 * gcol) * SBO;
+    const float4 *twt = reinterpret_cast<const float4 *>(sm + OFF_TW) + 16 * 64 * gcol + r;
+    const uint32_t amx_t = smem_u32(sm + OFF_AMX) + 32 * GT * grp + gt;      // this thread's cells, stride GT
 
     // ---- the three thread phases of one template --------------------------------
-    // Warp 0 issues each product (one elected lane, so the warp never diverges
-    // around an issue) right after the barrier that completes its operand.
-    const uint64_t dA1 = sdesc(smem_u32(sm + OFF_A1)), dA3 = sdesc(smem_u32(sm + OFF_A3)),
-                   dB = sdesc(smem_u32(sm + OFF_B));
-    // A: Z = X C (scaled) -> A1 (K-major), from ring buffer `b`
-    auto phase_a = [&](int b) {
-        // template values f = ka + 64 (8 blk + i) and f + 64, paired in the bank
-        const float4 *C = reinterpret_cast<const float4 *>(ring + b * L) + ka + 64 * 4 * blk;
-        uint32_t pr[8], pi[8];                                // [seg 0: 0..3 | seg 1: 4..7]
+    // The group's warp 0 issues each product (one elected lane, so the warp never
+    // diverges around an issue) right after the barrier that completes its operand.
+    const uint64_t dA = sdesc(smem_u32(opa)), dB = sdesc(smem_u32(sm + OFF_B));
+    const uint32_t td = tmem + 128 * (uint32_t)grp;           // the group's accumulator
+    // A: Z = X C (scaled) -> operand (K-major), from the group's template buffer
+    auto phase_a = [&]() {
+        // template values f = ka + 64 (16 blk + i) and f + 64, paired in the bank
+        const float4 *C = reinterpret_cast<const float4 *>(buf) + ka + 64 * 8 * blk;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float4 c = C[64 * i];
-            const float2 cr = make_float2(c.x, c.y), ci = make_float2(c.z, c.w);
+        for (int c = 0; c < 2; ++c) {
+            uint32_t x[32];
+            tmem_ld32(tx + 32 * c, x);
+            float4 cv[4];
 #pragma unroll
-            for (int s2 = 0; s2 < SEGS; ++s2) {
-                // two complex products per packed instruction
-                const float2 zr = sub2(mul2(xr[s2][i], cr), mul2(xi[s2][i], ci));
-                const float2 zi = fma2(xr[s2][i], ci, mul2(xi[s2][i], cr));
-                pr[4 * s2 + i] = pack2<PREC>(zr.x, zr.y);
-                pi[4 * s2 + i] = pack2<PREC>(zi.x, zi.y);
+            for (int i = 0; i < 4; ++i) cv[i] = C[64 * (4 * c + i)];
+            tmem_wait_ld32(x);
+            uint32_t pr[8], pi[8];                            // [seg 0: 0..3 | seg 1: 4..7]
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 cr = make_float2(cv[i].x, cv[i].y), ci = make_float2(cv[i].z, cv[i].w);
+#pragma unroll
+                for (int s2 = 0; s2 < SEGS; ++s2) {
+                    const uint32_t *xv = x + 16 * s2 + 4 * i;
+                    const float2 xr = make_float2(__uint_as_float(xv[0]), __uint_as_float(xv[1]));
+                    const float2 xi = make_float2(__uint_as_float(xv[2]), __uint_as_float(xv[3]));
+                    // two complex products per packed instruction
+                    const float2 zr = sub2(mul2(xr, cr), mul2(xi, ci));
+                    const float2 zi = fma2(xr, ci, mul2(xi, cr));
+                    pr[4 * s2 + i] = pack2<PREC>(zr.x, zr.y);
+                    pi[4 * s2 + i] = pack2<PREC>(zi.x, zi.y);
+                }
             }
+            sts128(a1_r0 + c * LBO, pr, 0);
+            sts128(a1_r0 + (8 + c) * LBO, pi, 0);
+            sts128(a1_r1 + c * LBO, pr, 4);
+            sts128(a1_r1 + (8 + c) * LBO, pi, 4);
         }
-        sts128(a1_r0, pr, 0);
-        sts128(a1_r0 + 8 * LBO, pi, 0);
-        sts128(a1_r1, pr, 4);
-        sts128(a1_r1 + 8 * LBO, pi, 4);
     };
-    // C: D1 -> twiddle -> A3 (MN-major)
+    // C: D -> twiddle -> operand (MN-major)
     auto phase_c = [&]() {
-        float ur[16], ui[16];
-        tmem_ld16x2(tmem + tlane + 16 * gcol, tmem + tlane + 64 + 16 * gcol, ur, ui);
-        uint32_t pr[8], pi[8];
 #pragma unroll
-        for (int i = 0; i < 16; i += 2) {
-            // cells i, i + 1 at once: packed complex product with their twiddles
-            const float4 w = twt[(i >> 1) * 64];
-            const float2 re = make_float2(ur[i], ur[i + 1]), im = make_float2(ui[i], ui[i + 1]);
-            const float2 wr = make_float2(w.x, w.y), wi = make_float2(w.z, w.w);
-            const float2 ore = sub2(mul2(re, wr), mul2(im, wi));
-            const float2 oim = fma2(re, wi, mul2(im, wr));
-            pr[i >> 1] = pack2<PREC>(ore.x, ore.y);
-            pi[i >> 1] = pack2<PREC>(oim.x, oim.y);
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t col = 32 * gcol + 16 * h;
+            float ur[16], ui[16];
+            tmem_ld16x2(td + tlane + col, td + tlane + 64 + col, ur, ui);
+            uint32_t pr[8], pi[8];
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) {
+                // cells i, i + 1 at once: packed complex product with their twiddles
+                const float4 w = twt[(8 * h + (i >> 1)) * 64];
+                const float2 re = make_float2(ur[i], ur[i + 1]), im = make_float2(ui[i], ui[i + 1]);
+                const float2 wr = make_float2(w.x, w.y), wi = make_float2(w.z, w.w);
+                const float2 ore = sub2(mul2(re, wr), mul2(im, wi));
+                const float2 oim = fma2(re, wi, mul2(im, wr));
+                pr[i >> 1] = pack2<PREC>(ore.x, ore.y);
+                pi[i >> 1] = pack2<PREC>(oim.x, oim.y);
+            }
+            const uint32_t to = a3_col + 2 * h * SBO;
+            sts128(to, pr, 0);
+            sts128(to + SBO, pr, 4);
+            sts128(to + 8 * LBO, pi, 0);
+            sts128(to + 8 * LBO + SBO, pi, 4);
         }
-        sts128(a3_col, pr, 0);
-        sts128(a3_col + SBO, pr, 4);
-        sts128(a3_col + 8 * LBO, pi, 0);
-        sts128(a3_col + 8 * LBO + SBO, pi, 4);
     };
-    // E: D3 -> power, running max, statistics, harmonic rows (search) or plane
+    // running maxima of the group's templates base .. into the stage-1 max-projection
+    auto flush_max = [&](int base) {
+        unsigned long long *M1 = itm->M1 + seg0 + r;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            if (i < nvalid) {
+                const int n = 64 * (32 * gcol + i);
+                const int am = sm[OFF_AMX + 32 * GT * grp + GT * i + gt];
+                // (a cell that is not a number under every template has no argmax: any valid position)
+                const int tw = __ldg(a.order + tb + min(2 * (base + am) + grp, nt - 1));
+                const unsigned long long packed = ((unsigned long long)__float_as_uint(mx[i] * psc) << 32) |
+                                                  (unsigned long long)(0xFFFFFFFFu - (unsigned)tw);
+                if (JERK_CHECK((int64_t)seg0 + n + r < bN, a.chk, kChkTcMaxProj)) atomicMax(M1 + n, packed);
+            }
+            mx[i] = -1.0f;
+        }
+    };
+    // E: D -> power, running max, statistics, harmonic rows (search) or plane
     // rows.
     // The running max and the statistics use |y|^2 before the segment's power
     // scale psc (a monotone factor), applied when they leave the CTA.  The max
-    // runs over all 16 cells: those past nvalid are never read back.  A warp
+    // runs over all cells: those past nvalid are never read back.  A warp
     // whose wait expired (`skip`) does none of it.
-    auto phase_e = [&](int k, int it, bool skip) {
+    auto phase_e = [&](int i0, bool skip) {
         if (skip) return;
-        float yr[16], yi[16];
-        tmem_ld16x2(tmem + tlane + 128 + 16 * gcol, tmem + tlane + 192 + 16 * gcol, yr, yi);
-        float P[16];
+        if constexpr (MODE == 0)
+            if (i0 > 0 && (i0 & (kFlush - 1)) == 0) flush_max(i0 - kFlush);
+        const TplMeta meta = tq[grp][i0 & 3];
+        float2 a2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, q2[2] = {a2[0], a2[0]};
 #pragma unroll
-        for (int i = 0; i < 16; i += 2) {
-            const float2 re = make_float2(yr[i], yr[i + 1]), im = make_float2(yi[i], yi[i + 1]);
-            const float2 p2 = fma2(re, re, mul2(im, im));    // two cells per packed instruction
-            P[i] = p2.x;
-            P[i + 1] = p2.y;
-        }
-        const int t = tq[k & 3].t;
-        if constexpr (MODE == 0) {
+        for (int h = 0; h < 2; ++h) {
+            const int cc = 2 * gcol + h;                      // cells n = 64 (16 cc + i) + r
+            const int nv = min(max(nvalid - 16 * h, 0), 16);
+            float yr[16], yi[16];
+            tmem_ld16x2(td + tlane + 16 * cc, td + tlane + 64 + 16 * cc, yr, yi);
+            float P[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                st_shared_u16_if(P[i] > mx[i], amx_t + 128 * i, (uint16_t)it);   // rare after the first templates
-                mx[i] = fmaxf(mx[i], P[i]);
+            for (int i = 0; i < 16; i += 2) {
+                const float2 re = make_float2(yr[i], yr[i + 1]), im = make_float2(yi[i], yi[i + 1]);
+                const float2 p2 = fma2(re, re, mul2(im, im));    // two cells per packed instruction
+                P[i] = p2.x;
+                P[i + 1] = p2.y;
             }
-            if constexpr (STATS) {
-                // four independent chains over the thread's cells (two packed
-                // pairs); cells outside the segment's valid range count as 0
-                float2 a2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, q2[2] = {a2[0], a2[0]};
-                if (nvalid == 16) {
+            if constexpr (MODE == 0) {
 #pragma unroll
-                    for (int i = 0; i < 16; i += 2) {
-                        const float2 p = make_float2(P[i], P[i + 1]);
-                        a2[(i >> 1) & 1] = add2(a2[(i >> 1) & 1], p);
-                        q2[(i >> 1) & 1] = fma2(p, p, q2[(i >> 1) & 1]);
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 16; i += 2) {
-                        const float2 p = make_float2(i < nvalid ? P[i] : 0.f, i + 1 < nvalid ? P[i + 1] : 0.f);
-                        a2[(i >> 1) & 1] = add2(a2[(i >> 1) & 1], p);
-                        q2[(i >> 1) & 1] = fma2(p, p, q2[(i >> 1) & 1]);
-                    }
+                for (int i = 0; i < 16; ++i) {
+                    max_arg(P[i], mx[16 * h + i], amx_t + GT * (16 * h + i), i0);
                 }
-                const float2 as = add2(a2[0], a2[1]), qs = add2(q2[0], q2[1]);
-                c1 += as.x + as.y;
-                c2 += qs.x + qs.y;
-                if ((it & 31) == 31) {
-                    // unscaled: the segment's scale is applied once, at the end
-                    add_f64_pair(&dacc[0][tid], &dacc[1][tid], c1, c2);
-                    c1 = c2 = 0.f;
-                }
-            }
-            // harmonic rows: cell q = q0 + 64 i (q0 = seg0 + 1024 gcol + r) is
-            // harmonic h of fundamental cell q / h when h | q; stored straight
-            // from registers (lanes hold consecutive cells)
-            const RowEntries &en = rent[k & 1];
-            const int ne = tq[k & 3].e1 - tq[k & 3].e0;
-            const int q0 = seg0 + 1024 * gcol + r;
-            if (ne > 0) {
-                // the rows hold scaled powers (P is not read again)
+                if constexpr (STATS) {
+                    // four independent chains over the thread's cells (two packed
+                    // pairs); cells outside the segment's valid range count as 0
+                    if (nv == 16) {
 #pragma unroll
-                for (int i = 0; i < 16; i += 2) {
-                    const float2 ps = mul2(make_float2(P[i], P[i + 1]), make_float2(psc, psc));
-                    P[i] = ps.x;
-                    P[i + 1] = ps.y;
-                }
-            }
-            for (int e = 0; e < ne; ++e) {
-                const int h = en.h[e];
-                float *dst = a.slots + en.off[e];
-                const int len = (int)en.len[e];
-                if ((h & (h - 1)) == 0) {
-                    // h = 1, 2, 4, 8 divides 64: all of this thread's cells are
-                    // harmonics of this h, or none is; cell i goes to row
-                    // position quo + i dq (dq = 64 / h) while that is below len.
-                    // The stride is a compile-time constant per h, so the 16
-                    // stores take immediate offsets from one address.
-                    const int lh = __ffs(h) - 1, ldq = 6 - lh;
-                    if ((q0 & (h - 1)) == 0) {
-                        const int quo = q0 >> lh;
-                        const int iend = quo >= len ? 0 : min(nvalid, (len - quo + (1 << ldq) - 1) >> ldq);
-                        float *d = dst + quo;
-                        auto rows16 = [&](auto ldqc) {
-                            constexpr int LDQ = decltype(ldqc)::value;
-                            if (iend == 16) {
+                        for (int i = 0; i < 16; i += 2) {
+                            const float2 p = make_float2(P[i], P[i + 1]);
+                            a2[(i >> 1) & 1] = add2(a2[(i >> 1) & 1], p);
+                            q2[(i >> 1) & 1] = fma2(p, p, q2[(i >> 1) & 1]);
+                        }
+                    } else {
 #pragma unroll
-                                for (int i = 0; i < 16; ++i)
-                                    if (JERK_CHECK(en.off[e] + quo + (i << LDQ) < a.slot_cap, a.chk, kChkTcRowStore))
-                                        d[i << LDQ] = P[i];
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 16; ++i)
-                                    if (i < iend &&
-                                        JERK_CHECK(en.off[e] + quo + (i << LDQ) < a.slot_cap, a.chk, kChkTcRowStore))
-                                        d[i << LDQ] = P[i];
-                            }
-                        };
-                        if (h == 1) rows16(std::integral_constant<int, 6>{});
-                        else if (h == 2) rows16(std::integral_constant<int, 5>{});
-                        else if (h == 4) rows16(std::integral_constant<int, 4>{});
-                        else rows16(std::integral_constant<int, 3>{});
-                    }
-                } else {
-                    // h = 3, 5, 6, 7: quotient and remainder stepped by 64 per cell
-                    int quo = q0 / h, rem = q0 - quo * h;
-                    const int dq = 64 / h, dr = 64 - dq * h;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        if (i < nvalid && rem == 0 && quo < len &&
-                            JERK_CHECK(en.off[e] + quo < a.slot_cap, a.chk, kChkTcRowStore))
-                            dst[quo] = P[i];
-                        quo += dq;
-                        rem += dr;
-                        if (rem >= h) {
-                            rem -= h;
-                            quo += 1;
+                        for (int i = 0; i < 16; i += 2) {
+                            const float2 p = make_float2(i < nv ? P[i] : 0.f, i + 1 < nv ? P[i + 1] : 0.f);
+                            a2[(i >> 1) & 1] = add2(a2[(i >> 1) & 1], p);
+                            q2[(i >> 1) & 1] = fma2(p, p, q2[(i >> 1) & 1]);
                         }
                     }
                 }
-            }
-        } else {
-            const int64_t row0 = (int64_t)(t - a.t0) * bN + seg0;
-            float *prow = a.plane + row0;
+                // harmonic rows: cell q = q0 + 64 i (q0 = seg0 + 1024 cc + r) is
+                // harmonic h of fundamental cell q / h when h | q; stored straight
+                // from registers (lanes hold consecutive cells)
+                const RowEntries &en = rent[grp][i0 & 1];
+                const int ne = meta.e1 - meta.e0;
+                const int q0 = seg0 + 1024 * cc + r;
+                if (ne > 0) {
+                    // the rows hold scaled powers (P is not read again)
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (i < nvalid &&
-                    JERK_CHECK(row0 + 64 * (16 * gcol + i) + r < a.plane_len, a.chk, kChkTcPlaneStore))
-                    prow[64 * (16 * gcol + i) + r] = P[i] * psc;
+                    for (int i = 0; i < 16; i += 2) {
+                        const float2 ps = mul2(make_float2(P[i], P[i + 1]), make_float2(psc, psc));
+                        P[i] = ps.x;
+                        P[i + 1] = ps.y;
+                    }
+                }
+                for (int e = 0; e < ne; ++e) {
+                    const int hh = en.h[e];
+                    float *dst = a.slots + en.off[e];
+                    const int len = (int)en.len[e];
+                    if ((hh & (hh - 1)) == 0) {
+                        // h = 1, 2, 4, 8 divides 64: all of this thread's cells are
+                        // harmonics of this h, or none is; cell i goes to row
+                        // position quo + i dq (dq = 64 / h) while that is below len.
+                        // The stride is a compile-time constant per h, so the 16
+                        // stores take immediate offsets from one address.
+                        const int lh = __ffs(hh) - 1, ldq = 6 - lh;
+                        if ((q0 & (hh - 1)) == 0) {
+                            const int quo = q0 >> lh;
+                            const int iend = quo >= len ? 0 : min(nv, (len - quo + (1 << ldq) - 1) >> ldq);
+                            float *d = dst + quo;
+                            auto rows16 = [&](auto ldqc) {
+                                constexpr int LDQ = decltype(ldqc)::value;
+                                if (iend == 16) {
+#pragma unroll
+                                    for (int i = 0; i < 16; ++i)
+                                        if (JERK_CHECK(en.off[e] + quo + (i << LDQ) < a.slot_cap, a.chk, kChkTcRowStore))
+                                            d[i << LDQ] = P[i];
+                                } else {
+#pragma unroll
+                                    for (int i = 0; i < 16; ++i)
+                                        if (i < iend &&
+                                            JERK_CHECK(en.off[e] + quo + (i << LDQ) < a.slot_cap, a.chk, kChkTcRowStore))
+                                            d[i << LDQ] = P[i];
+                                }
+                            };
+                            if (hh == 1) rows16(std::integral_constant<int, 6>{});
+                            else if (hh == 2) rows16(std::integral_constant<int, 5>{});
+                            else if (hh == 4) rows16(std::integral_constant<int, 4>{});
+                            else rows16(std::integral_constant<int, 3>{});
+                        }
+                    } else {
+                        // h = 3, 5, 6, 7: quotient and remainder stepped by 64 per cell
+                        int quo = q0 / hh, rem = q0 - quo * hh;
+                        const int dq = 64 / hh, dr = 64 - dq * hh;
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            if (i < nv && rem == 0 && quo < len &&
+                                JERK_CHECK(en.off[e] + quo < a.slot_cap, a.chk, kChkTcRowStore))
+                                dst[quo] = P[i];
+                            quo += dq;
+                            rem += dr;
+                            if (rem >= hh) {
+                                rem -= hh;
+                                quo += 1;
+                            }
+                        }
+                    }
+                }
+            } else {
+                const int64_t row0 = (int64_t)(meta.t - a.t0) * bN + seg0;
+                float *prow = a.plane + row0;
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (i < nv && JERK_CHECK(row0 + 64 * (16 * cc + i) + r < a.plane_len, a.chk, kChkTcPlaneStore))
+                        prow[64 * (16 * cc + i) + r] = P[i] * psc;
+            }
+        }
+        if constexpr (MODE == 0 && STATS) {
+            const float2 as = add2(a2[0], a2[1]), qs = add2(q2[0], q2[1]);
+            c1 += as.x + as.y;
+            c2 += qs.x + qs.y;
+            if ((i0 & 31) == 31) {
+                // unscaled: the segment's scale is applied once, at the end
+                add_f64_pair(&dacc[0][tid], &dacc[1][tid], c1, c2);
+                c1 = c2 = 0.f;
+            }
         }
     };
 
-    // ---- software pipeline over the group's templates ------------------------------
-    // iteration it:  C(it) | A(it+1) with step 3 of it issued || E(it) with step 1
-    // of it+1 issued, so each product runs while the threads work on the other.
-    const int nt = te - tb;
+    // ---- the group's templates ---------------------------------------------------
+    // A | step 1 | C | step 3 | E, one after another; the other group's phases and
+    // products run in the waits.  `fail` is warp-uniform after each wait and
+    // group-uniform after each named_any; a group leaves only there, so all its
+    // warps take the same barriers.
     bool fail = !mbar_wait_bounded(&cbar, 0);
     fail = __any_sync(0xffffffffu, fail);
-    if (nt > 0) {
-        if (!fail) fail = !mbar_wait_bounded(&full[0], 0);
+    for (int i = 0; i < ng; ++i) {
+        const int it = 2 * i + grp;                           // position in the CTA's list
+        if (!fail) fail = !mbar_wait_bounded(&full[grp], (uint32_t)i & 1u);
         fail = __any_sync(0xffffffffu, fail);
-        if (!fail) phase_a(0);
+        // (the operand is free: step 3 of the last template was waited for)
+        if (!fail) phase_a();
+        tc_fence_before();                                    // E's reads of D, before step 1 writes it
         fence_async_smem();
-        fail = __syncthreads_or(fail);
-        if (!fail && warp == 0) {
+        fail = named_any(1 + grp, GT, fail);
+        if (fail) break;
+        if (gwarp == 0) {
             tc_fence_after();
-            mma_tile_warp<PREC, false>(tmem, dA1, dB);
-            mma_commit_warp(&mbar1);
+            mma_tile_warp<PREC, false>(td, dA, dB);
+            if (!inject_at(a, 2, it)) mma_commit_warp(&mbar1[grp]);
         }
-        if (!fail && tid == 32 && nt > 2) {                    // buffer 0 is read: template 2 next
-            issued[0] += 1;
-            bulk_load(ring, a.bank + (int64_t)tc_bank_row<ROWS>(a, tb + 2) * L, (uint32_t)(L * sizeof(float2)),
-                      &full[0]);
+        if (gt == 32 && it + 2 < nt && !inject_at(a, 1, it + 2)) {   // the template is read: the group's next
+            issued[grp] += 1;
+            bulk_load(buf, a.bank + (int64_t)tc_bank_row<ROWS>(a, tb + it + 2) * L, (uint32_t)(L * sizeof(float2)),
+                      &full[grp]);
         }
-    }
-    // `fail` is warp-uniform after each wait and CTA-uniform after each
-    // __syncthreads_or; the loop is left only there, so every warp takes the
-    // same barriers.
-    for (int it = 0; it < nt; ++it) {
-        // C(it): step 1 of template it has landed in D1
-        if (!fail) fail = !mbar_wait_bounded(&mbar1, (uint32_t)it & 1u);
+        fail = !mbar_wait_bounded(&mbar1[grp], (uint32_t)i & 1u);
         fail = __any_sync(0xffffffffu, fail);
         tc_fence_after();
         if (!fail) phase_c();
-        if (warp == 2) cp_async_wait_all();                   // the metadata issued last template
+        if (gwarp == 2) cp_async_wait_all();                  // the metadata issued last template
         tc_fence_before();
         fence_async_smem();
-        if (__syncthreads_or(fail)) {
-            fail = true;
-            break;
+        fail = named_any(1 + grp, GT, fail);
+        if (fail) break;
+        if (gwarp == 0) {
+            tc_fence_after();
+            mma_tile_warp<PREC, true>(td, dA, dB);
+            if (!inject_at(a, 3, it)) mma_commit_warp(&mbar3[grp]);
         }
-        if (warp == 2) {
+        if (gwarp == 2) {
             // Metadata pipeline (no L2-latency load between a product and the
-            // epilogue that needs it): t of template k + 3, then (e0, e1) of
-            // k + 2, then the slot entries of k + 1.  Every thread is past E of
+            // epilogue that needs it): t of the group's template i + 3, then (e0, e1)
+            // of i + 2, then the slot entries of i + 1.  Every thread is past E of
             // the previous template, the last reader of the slots written here.
-            const int k = tb + it;
             if (lane == 0) {
-                if (k + 3 < te) cp_async<4>(&tq[(k + 3) & 3].t, a.order + k + 3);
-                if (MODE == 0 && k + 2 < te) {
-                    const int t2 = tq[(k + 2) & 3].t;
-                    cp_async<4>(&tq[(k + 2) & 3].e0, a.slot_beg + t2);
-                    cp_async<4>(&tq[(k + 2) & 3].e1, a.slot_beg + t2 + 1);
+                if (i + 3 < ng) cp_async<4>(&tq[grp][(i + 3) & 3].t, a.order + tb + it + 6);
+                if (MODE == 0 && i + 2 < ng) {
+                    const int t2 = tq[grp][(i + 2) & 3].t;
+                    cp_async<4>(&tq[grp][(i + 2) & 3].e0, a.slot_beg + t2);
+                    cp_async<4>(&tq[grp][(i + 2) & 3].e1, a.slot_beg + t2 + 1);
                 }
             }
-            if (MODE == 0 && k + 1 < te) {
-                const TplMeta m1 = tq[(k + 1) & 3];
+            if (MODE == 0 && i + 1 < ng) {
+                const TplMeta m1 = tq[grp][(i + 1) & 3];
                 if (lane < m1.e1 - m1.e0) {
                     const int e = m1.e0 + lane;
-                    RowEntries &en = rent[(k + 1) & 1];
+                    RowEntries &en = rent[grp][(i + 1) & 1];
                     cp_async<4>(&en.h[lane], a.slot_h + e);
                     cp_async<8>(&en.off[lane], itm->slot_off + e);
                     cp_async<8>(&en.len[lane], itm->slot_len + e);
@@ -614,62 +679,19 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
             }
             cp_async_commit();
         }
-        if (warp == 0) {
-            // step 3 of template it (its operand A3 is complete)
-            tc_fence_after();
-            mma_tile_warp<PREC, true>(tmem + 128, dA3, dB);
-            if (!inject_at(a, 3, it)) mma_commit_warp(&mbar3);
-        }
-        const bool more = it + 1 < nt;
-        if (more) {
-            // A(it + 1) while step 3 of template it runs
-            const int b = (it + 1) & 1;
-            fail = !mbar_wait_bounded(&full[b], (uint32_t)((it + 1) >> 1) & 1u);
-            fail = __any_sync(0xffffffffu, fail);
-            if (!fail) phase_a(b);
-            fence_async_smem();
-            if (__syncthreads_or(fail)) {
-                fail = true;
-                break;
-            }
-            if (tid == 32 && it + 3 < nt && !inject_at(a, 1, it + 3)) {   // buffer b is read: template it + 3 next
-                issued[b] += 1;
-                bulk_load(ring + b * L, a.bank + (int64_t)tc_bank_row<ROWS>(a, tb + it + 3) * L,
-                          (uint32_t)(L * sizeof(float2)), &full[b]);
-            }
-            if (warp == 0) {
-                // step 1 of template it + 1 (queued behind step 3 of it)
-                tc_fence_after();
-                mma_tile_warp<PREC, false>(tmem, dA1, dB);
-                if (!inject_at(a, 2, it + 1)) mma_commit_warp(&mbar1);
-            }
-        }
-        // E(it): step 3 of template it has landed in D3; step 1 of it + 1 runs meanwhile
-        fail = !mbar_wait_bounded(&mbar3, (uint32_t)it & 1u);
+        fail = !mbar_wait_bounded(&mbar3[grp], (uint32_t)i & 1u);
         fail = __any_sync(0xffffffffu, fail);
         tc_fence_after();
-        phase_e(tb + it, it, fail);
-        tc_fence_before();
+        phase_e(i, fail);
     }
-    if (warp == 2) cp_async_wait_all();                       // no copy in flight past the loop
+    if (gwarp == 2) cp_async_wait_all();                      // no copy in flight past the loop
+    tc_fence_before();
     fail = __syncthreads_or(fail);
 
     // ---- epilogue -----------------------------------------------------------------
     if (fail && tid == 0) atomicExch(a.err, 1);
     if constexpr (MODE == 0) {
-        if (!fail && tb < te) {
-            unsigned long long *M1 = itm->M1;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                if (i < nvalid) {
-                    const int n = 64 * (16 * gcol + i) + r;
-                    const int tw = __ldg(a.order + tb + amx_s[seg * L + n]);
-                    const unsigned long long packed = ((unsigned long long)__float_as_uint(mx[i] * psc) << 32) |
-                                                      (unsigned long long)(0xFFFFFFFFu - (unsigned)tw);
-                    if (JERK_CHECK((int64_t)seg0 + n < bN, a.chk, kChkTcMaxProj)) atomicMax(M1 + seg0 + n, packed);
-                }
-            }
-        }
+        if (!fail && ng > 0) flush_max((ng - 1) / kFlush * kFlush);
         if constexpr (STATS) {
             double d1 = (dacc[0][tid] + (double)c1) * (double)psc;
             double d2 = (dacc[1][tid] + (double)c2) * ((double)psc * (double)psc);
@@ -696,15 +718,15 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
     }
     if (tid == 0) {
         // never leave with a bulk copy still writing into this CTA's shared memory
-        for (int b = 0; b < 2; ++b)
-            if (issued[b] > 0) mbar_wait_bounded(&full[b], (uint32_t)(issued[b] - 1) & 1u);
+        for (int g = 0; g < 2; ++g)
+            if (issued[g] > 0) mbar_wait_bounded(&full[g], (uint32_t)(issued[g] - 1) & 1u);
         mbar_wait_bounded(&cbar, 0);
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+        tmem_dealloc_warp(tmem, TMEM_COLS);
     }
 }
 

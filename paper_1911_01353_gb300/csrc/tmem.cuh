@@ -1,4 +1,4 @@
-// Tensor memory as per-thread storage for the FP32 filter's constant factors.
+// Tensor memory as per-thread storage for the filters' constant factors.
 //
 // Each SM has 256 KB of tensor memory (128 lanes x 512 columns of 32 bits),
 // read by tcgen05.ld on its own path, not through the shared-memory pipe.
@@ -6,8 +6,8 @@
 // thread, so a thread can keep private words there: warps w, w + 4, w + 8,
 // w + 12 share a lane range and take disjoint column ranges.  The FP32 filter
 // keeps the twiddle factors of its inverse transform there (the same for
-// every template), which takes their reads off the shared-memory pipe that
-// bounds it.
+// every template), both filters the spectrum values a thread multiplies, which
+// takes their reads off the shared-memory pipe and out of the registers.
 #pragma once
 
 #include <stdint.h>
@@ -60,6 +60,49 @@ __device__ __forceinline__ void tmem_wait_ld8(uint32_t (&r)[8]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
                  :
+                 : "memory");
+}
+
+// the same for 32 columns
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, "
+                 "%8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, "
+                 "%24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                   "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+                   "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+                   "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld32(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                   "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
+                   "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+                 :
+                 : "memory");
+}
+
+// two FP64 values in 4 consecutive columns of this thread's lane (warp-collective, waited for)
+__device__ __forceinline__ void tmem_ld_f64x2(uint32_t taddr, double &a, double &b) {
+    uint32_t r[4];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr)
+                 : "memory");
+    a = __hiloint2double((int)r[1], (int)r[0]);
+    b = __hiloint2double((int)r[3], (int)r[2]);
+}
+__device__ __forceinline__ void tmem_st_f64x2(uint32_t taddr, double a, double b) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n\ttcgen05.wait::st.sync.aligned;" ::"r"(
+                     taddr),
+                 "r"((uint32_t)__double2loint(a)), "r"((uint32_t)__double2hiint(a)),
+                 "r"((uint32_t)__double2loint(b)), "r"((uint32_t)__double2hiint(b))
                  : "memory");
 }
 
