@@ -95,9 +95,9 @@ def conv_flops_per_cell(L, V):
     return (5.0 * L * math.log2(L) + 6.0 * L + 3.0 * V) / V
 
 
-def kernel_hash(main="conv.cu"):
+def kernel_hash(main="conv_pair.cu"):
     h = hashlib.sha256()
-    for f in (main, "fft.cuh", "device_sync.cuh", "rows.cuh"):
+    for f in (main, "fft.cuh", "pair.cuh", "tmem.cuh", "device_sync.cuh", "rows.cuh"):
         with open(os.path.join(ROOT, "paper_1911_01353_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -121,7 +121,7 @@ def recorded_traffic(L, alg_bytes, precision=0):
     (``conv_algorithmic_bytes``).  Returns (bytes, note), or (None, why) when
     no record was taken on the current kernel sources."""
     name = TRAFFIC_FILES[precision]
-    main = "conv.cu" if precision == 0 else "conv_tc.cu"
+    main = "conv_pair.cu" if precision == 0 else "conv_tc.cu"
     path = os.path.join(ROOT, "profiles", name)
     if not os.path.exists(path):
         return None, "no record"
@@ -161,7 +161,7 @@ def recorded_limiter(L, precision=0):
             if ":" in line and not line.startswith("#"):
                 k, v = line.split(":", 1)
                 vals[k.strip()] = v.strip()
-    main = "conv.cu" if precision == 0 else "conv_tc.cu"
+    main = "conv_pair.cu" if precision == 0 else "conv_tc.cu"
     if vals.get("kernel_sha") != kernel_hash(main) or int(vals.get("seg_len", 0)) != L:
         return None
     out = {}
@@ -621,7 +621,7 @@ def main():
     traffic, traffic_note = recorded_traffic(L, alg_bytes, a.precision)
     peaks, peaks_src = peaks_file()
 
-    roof = {"bound": "alu", "kernel": "conv_kernel (fused FFT-multiply-IFFT-power)",
+    roof = {"bound": "alu", "kernel": "conv_pair_kernel (fused FFT-multiply-IFFT-power)",
             "achieved": achieved, "peak": peak_alu, "unit": "TFLOP/s",
             "frac": achieved / peak_alu, "traffic": traffic, "traffic_note": traffic_note,
             "limiter": recorded_limiter(L, 0),
@@ -699,7 +699,7 @@ def main():
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(spec.nbytes),
                     "d2h_bytes_per_step": 8 + 24 * ncand},
-            "gpu_launches": 5 * a.steps,
+            "gpu_launches": 7 * a.steps,
             "clocks": clk,
         }
         if accuracy is not None:

@@ -212,7 +212,9 @@ constexpr int kTcBankPair = 64;
 cudaError_t launch_twiddles64(double2 *tw, int L, cudaStream_t st);
 cudaError_t launch_conv(int log2L, int mode, bool stats, const ConvArgs &a, int n_ctas, cudaStream_t st);
 cudaError_t launch_conv_tc(int precision, int mode, bool stats, const ConvArgs &a, int n_ctas, cudaStream_t st);
-int conv_segs_per_cta(int log2L);
+int conv_segs_per_cta(int log2L, int precision);
+constexpr int kPairSegs = 3;         // segments of a CTA of the L = 4096 filter (conv_pair.cu)
+cudaError_t launch_conv_pair(int mode, bool stats, const ConvArgs &a, int n_ctas, cudaStream_t st);
 cudaError_t launch_harmonic(const HarmArgs &a, int64_t blocks, bool stats, cudaStream_t st);
 int harmonic_cells_per_block();
 cudaError_t launch_finalise_stats(const ItemDesc *items, int n_items, const double *part1, const double *partH,

@@ -50,6 +50,9 @@ __device__ __forceinline__ float scaled(float f, double scale, float sh, float s
 // sums and extrema over the W warps of a block of bins
 template <int W>
 struct BlockOf {
+    static __device__ __forceinline__ void sync() {
+        if constexpr (W > 1) __syncthreads(); else __syncwarp();
+    }
     static __device__ __forceinline__ unsigned add(unsigned x) {
         x = __reduce_add_sync(0xffffffffu, x);
         if constexpr (W > 1) x = across(x, [](unsigned a, unsigned b) { return a + b; });
@@ -96,11 +99,12 @@ __global__ void __launch_bounds__(32 * W) normalise_kernel(NormArgs a, int B) {
     const float2 *in = a.in[item] + s0;
     float2 *out = a.out[item] + s0;
     const int tid = threadIdx.x;
-    // FP32 powers, or FP64 ones rounded to FP32 (exact: both keep the order of the FP64 powers)
     unsigned key[KPT];
     const unsigned rank = (unsigned)(nb - 1) / 2;
     unsigned lo, hi, n_lo;
-    auto bisect = [&](bool exact) {
+    // pass 0: FP32 powers; pass 1, where those are too small or too large: FP64
+    // powers rounded to FP32, which keeps their order
+    for (int pass = 0;; ++pass) {
         lo = ~0u;
         hi = 0u;
 #pragma unroll
@@ -109,8 +113,8 @@ __global__ void __launch_bounds__(32 * W) normalise_kernel(NormArgs a, int B) {
             key[i] = ~0u;                                     // above every power: never counted
             if (k < nb) {
                 const float2 f = in[k];
-                key[i] = exact ? __float_as_uint((float)__longlong_as_double((long long)power_key(f)))
-                               : __float_as_uint(fmaf(f.x, f.x, f.y * f.y));
+                key[i] = __float_as_uint(fmaf(f.x, f.x, f.y * f.y));
+                if (pass) key[i] = __float_as_uint((float)__longlong_as_double((long long)power_key(f)));
                 lo = min(lo, key[i]);
                 hi = max(hi, key[i]);
             }
@@ -139,10 +143,8 @@ __global__ void __launch_bounds__(32 * W) normalise_kernel(NormArgs a, int B) {
                 n_lo = c;
             }
         }
-    };
-    bisect(false);
-    {
-        // narrow [lo, hi] to the one key of that rank: the smallest in it at or above lo
+        if (pass) break;
+        // the one key of that rank: the smallest in [lo, hi]
         unsigned v = ~0u;
 #pragma unroll
         for (int i = 0; i < KPT; ++i)
@@ -158,33 +160,62 @@ __global__ void __launch_bounds__(32 * W) normalise_kernel(NormArgs a, int B) {
 #pragma unroll
             for (int i = 0; i < KPT; ++i) c += key[i] < lo ? 1u : 0u;
             n_lo = BlockOf<W>::add(c);
-        } else {
-            bisect(true);
+            break;
         }
     }
-    // among the bins in [lo, hi], by FP64 powers: their range, then by counting again if it is wider than one value
-    unsigned long long lo64 = ~0ull, hi64 = 0ull;
+    // among the bins in [lo, hi], listed, by their FP64 powers: the one with at
+    // most rank - n_lo others below it and more than that not above it
+    constexpr int LIST = 64;
+    __shared__ unsigned long long list[LIST], med64;
+    __shared__ int listed;
+    if (tid == 0) listed = 0;
+    BlockOf<W>::sync();
 #pragma unroll
-    for (int i = 0; i < KPT; ++i) {
+    for (int i = 0; i < KPT; ++i)
         if (key[i] >= lo && key[i] <= hi) {
-            const unsigned long long v = power_key(in[tid + NT * i]);
-            lo64 = v < lo64 ? v : lo64;
-            hi64 = v > hi64 ? v : hi64;
+            const int at = atomicAdd(&listed, 1);
+            if (at < LIST) list[at] = power_key(in[tid + NT * i]);
         }
-    }
-    lo64 = BlockOf<W>::low64(lo64);
-    hi64 = BlockOf<W>::high64(hi64);
-    while (lo64 < hi64) {
-        const unsigned long long mid = lo64 + (hi64 - lo64) / 2;
-        unsigned c = 0;
+    BlockOf<W>::sync();
+    const int n_list = listed;
+    unsigned long long lo64;
+    if (n_list <= LIST) {
+        for (int i = tid; i < n_list; i += NT) {
+            unsigned below = 0, equal = 0;
+            for (int q = 0; q < n_list; ++q) {
+                below += list[q] < list[i] ? 1u : 0u;
+                equal += list[q] == list[i] ? 1u : 0u;
+            }
+            if (below <= rank - n_lo && rank - n_lo < below + equal) med64 = list[i];
+        }
+        BlockOf<W>::sync();
+        lo64 = med64;
+    } else {
+        // many equal FP32 powers: bisect the FP64 ones
+        unsigned long long hi64 = 0ull;
+        lo64 = ~0ull;
 #pragma unroll
-        for (int i = 0; i < KPT; ++i)
-            if (key[i] >= lo && key[i] <= hi) c += power_key(in[tid + NT * i]) <= mid ? 1u : 0u;
-        c = BlockOf<W>::add(c);
-        if (c > rank - n_lo)
-            hi64 = mid;
-        else
-            lo64 = mid + 1;
+        for (int i = 0; i < KPT; ++i) {
+            if (key[i] >= lo && key[i] <= hi) {
+                const unsigned long long v = power_key(in[tid + NT * i]);
+                lo64 = v < lo64 ? v : lo64;
+                hi64 = v > hi64 ? v : hi64;
+            }
+        }
+        lo64 = BlockOf<W>::low64(lo64);
+        hi64 = BlockOf<W>::high64(hi64);
+        while (lo64 < hi64) {
+            const unsigned long long mid = lo64 + (hi64 - lo64) / 2;
+            unsigned c = 0;
+#pragma unroll
+            for (int i = 0; i < KPT; ++i)
+                if (key[i] >= lo && key[i] <= hi) c += power_key(in[tid + NT * i]) <= mid ? 1u : 0u;
+            c = BlockOf<W>::add(c);
+            if (c > rank - n_lo)
+                hi64 = mid;
+            else
+                lo64 = mid + 1;
+        }
     }
     const double med = __longlong_as_double((long long)lo64);
     const double scale = med > 0.0 ? 1.0 / sqrt(med / 0.69314718055994530942) : 1.0;

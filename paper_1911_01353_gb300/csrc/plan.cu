@@ -173,6 +173,47 @@ int tpg_for(const jerk_plan_s *pl, int nseg, int nt) {
     return (int)std::max<int64_t>(tpg, 1);
 }
 
+// Templates per CTA of a search of n bins: whole groups, or equal parts of at
+// least kMinChunk templates where those take fewer steps.  A step is one
+// template of a CTA; setting one up takes about kSetup of them, and one CTA runs
+// per SM at a time, so whole waves count (700 001 bins, 3131 templates in four
+// groups: 508 CTAs of up to 1024 templates are four waves, the last a third full,
+// 10.40 ms; in parts 9.08).  The groups themselves stay: they fix the bank's rows and,
+// in reduced precision, where the 16-bit roundings fall.  A spectrum that does
+// not fill the chip with whole groups keeps them, since in a batch others fill
+// it.  The rule sees the spectrum's length alone, so its statistics are added in
+// the same order in every batch.
+constexpr int kMinChunk = 32, kSetup = 5;
+
+// parts a group of the plan can be cut into (sizing of the launch tables and partials)
+int max_parts(const jerk_plan_s *pl) {
+    int most = 1;
+    for (const auto &g : pl->groups) most = std::max(most, g.te - g.tb);
+    return std::max(1, most / kMinChunk);
+}
+
+int chunk_for(const jerk_plan_s *pl, int64_t n) {
+    const int64_t bN = (int64_t)pl->b * n;
+    const int segs = conv_segs_per_cta(pl->log2L, pl->prm.precision);
+    int most = 1;
+    for (const auto &g : pl->groups) most = std::max(most, g.te - g.tb);
+    int best = most;
+    int64_t best_cost = INT64_MAX;
+    for (int parts = 1; parts <= max_parts(pl); ++parts) {
+        const int c = (most + parts - 1) / parts;
+        int64_t ctas = 0;
+        for (const auto &g : pl->groups)
+            ctas += ((bN + g.V - 1) / g.V + segs - 1) / segs * ((g.te - g.tb + c - 1) / c);
+        if (parts == 1 && ctas < pl->sms) break;
+        const int64_t cost = (ctas + pl->sms - 1) / pl->sms * (c + kSetup);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
 // Group templates by filter half-width: sort by (m_t, t), cut into runs of
 // `tpg`, process each run in ascending t (so ties keep the lowest t).  A
 // group's tap offset is b * max(m_t) and its segment length L - 2 b max(m_t).
@@ -204,7 +245,7 @@ void build_groups(jerk_plan_s *pl, int tpg) {
 // conv CTAs one spectrum of n bins needs
 int64_t ctas_for(const jerk_plan_s *pl, int64_t n) {
     const int64_t bN = (int64_t)pl->b * n;
-    const int segs = conv_segs_per_cta(pl->log2L);
+    const int segs = conv_segs_per_cta(pl->log2L, pl->prm.precision);
     int64_t c = 0;
     for (const auto &x : pl->groups) c += ((bN + x.V - 1) / x.V + segs - 1) / segs;
     return c;
@@ -374,7 +415,7 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
     h.rows.clear();
     h.tl.clear();
     int64_t spec = 0, m[JERK_MAX_STAGES] = {0, 0, 0, 0};
-    const int segs = conv_segs_per_cta(pl->log2L);
+    const int segs = conv_segs_per_cta(pl->log2L, pl->prm.precision);
     for (int i = 0; i < count; ++i) {
         const int zs = !zm.empty() ? zm[i] : pl->prm.zmax, ws = !zm.empty() ? wm[i] : pl->prm.wmax;
         const int64_t bN = (int64_t)pl->b * n[i];
@@ -395,6 +436,7 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
         // conv work: this spectrum's (group, segment range) entries, item-major;
         // a sub-grid keeps, per group, the templates inside it (positions into `rows`)
         int64_t nt_item = 0;
+        const int chunk = chunk_for(pl, n[i]);
         // a partial search: templates outside the range that make a row of a range fundamental
         std::vector<char> extra;
         if (range) {
@@ -424,10 +466,14 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
                     if (w.te == w.tb) continue;
                 }
                 if (part == 0) nt_item += w.te - w.tb;
-                w.cta0 = (int32_t)L.total_ctas;
                 w.item = i;
-                h.work.push_back(w);
-                L.total_ctas += ((bN + g.V - 1) / g.V + segs - 1) / segs;
+                for (int tb = w.tb, te = w.te; tb < te; tb = w.te) {
+                    w.tb = tb;
+                    w.te = te - tb > chunk ? tb + chunk : te;
+                    w.cta0 = (int32_t)L.total_ctas;
+                    h.work.push_back(w);
+                    L.total_ctas += ((bN + g.V - 1) / g.V + segs - 1) / segs;
+                }
             }
         }
         L.item_cta0[i + 1] = L.total_ctas;
@@ -559,7 +605,7 @@ jerk_status transient_layout(jerk_plan_s *pl, const std::vector<int64_t> &n, con
     if (!tt.d_buf) {
         // capacity: max_batch items, each with every group, entry, fundamental and template
         const size_t mb = (size_t)pl->max_batch;
-        tt.cap_work = (int64_t)(mb * pl->groups.size() + 1);
+        tt.cap_work = (int64_t)(mb * pl->groups.size() * max_parts(pl) + 1);
         tt.cap_ent = (int64_t)(mb * std::max(pl->n_entries, 1));
         tt.cap_fund = (int64_t)(mb * std::max(pl->n_fund, 1));
         tt.cap_rows = (int64_t)(mb * pl->T);
@@ -855,7 +901,7 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
     // (rows, CTAs and harmonic blocks grow with n; each extra spectrum adds rounding)
     pl->slot_cap = item_rows(pl, N, params->zmax, params->wmax, 0, nullptr, nullptr, nullptr, nullptr, nullptr) +
                    (int64_t)pl->max_batch * 32 * std::max(1, pl->n_fund * JERK_MAX_HARMONIC);
-    const int64_t conv_blocks = ctas_for(pl, N) + (int64_t)pl->max_batch * (int64_t)pl->groups.size();
+    const int64_t conv_blocks = (ctas_for(pl, N) + (int64_t)pl->max_batch * (int64_t)pl->groups.size()) * max_parts(pl);
     // (a spectrum's harmonic blocks are at most one per SM more than its blocks of cells)
     const int64_t harm_blocks = harm_nx_for(pl, N) + (int64_t)pl->max_batch *
                                 (1 + std::min<int64_t>(pl->sms, (int64_t)(pl->n_fund / 8 + 1) * (harm_nx_for(pl, N) + 1)));
@@ -1213,15 +1259,18 @@ jerk_status jerk_plane(jerk_plan pl, const void *d_spec, int64_t n, int32_t t0, 
     // whole bank for 64 of 12 261 templates at 2^18 bins took 12.5 ms, this 0.15 ms
     int64_t first = -1, last = 0, at = 0;
     const int64_t bN = (int64_t)pl->b * n;
-    const int segs = conv_segs_per_cta(pl->log2L);
+    const int segs = conv_segs_per_cta(pl->log2L, pl->prm.precision), chunk = chunk_for(pl, n);
     for (const auto &g : pl->groups) {
-        const int64_t end = at + ((bN + g.V - 1) / g.V + segs - 1) / segs;
-        const auto k = std::lower_bound(pl->order.begin() + g.tb, pl->order.begin() + g.te, t0);
-        if (k != pl->order.begin() + g.te && *k < t0 + nt) {
-            if (first < 0) first = at;
-            last = end;
+        for (int tb = g.tb, te; tb < g.te; tb = te) {
+            te = g.te - tb > chunk ? tb + chunk : g.te;
+            const int64_t end = at + ((bN + g.V - 1) / g.V + segs - 1) / segs;
+            const auto k = std::lower_bound(pl->order.begin() + tb, pl->order.begin() + te, t0);
+            if (k != pl->order.begin() + te && *k < t0 + nt) {
+                if (first < 0) first = at;
+                last = end;
+            }
+            at = end;
         }
-        at = end;
     }
     a.cta_base = (int32_t)first;
     const int n_ctas = (int)(last - first);
