@@ -26,10 +26,11 @@
 // than with one complex value per register pair and 256 threads per segment).
 // Filter alone, bank of 12 261 templates, 2^21 bins, stages 1-2-4-8: 118.6 ->
 // 106.4 ms; 3131 templates, 700 001 bins: 10.37 -> 9.08 ms; six requests on the
-// bank of 27 391 templates, stage 1: 10.75 -> 9.28 ms.  Four segments of four
-// warps (maxima in tensor memory, pass-1 twiddles in shared memory, rows staged
-// in the exchange buffer) were 1 % faster at 2^21 bins but 5 % slower on the
-// requests and 27 % on short spectra, whose segments fill fewer CTAs: not kept.
+// bank of 27 391 templates, stage 1: 10.75 -> 9.28 ms.  Four segments a CTA
+// were not faster: as four of four warps (maxima in tensor memory, pass-1
+// twiddles in shared memory, rows staged in the exchange buffer) 27 % slower on
+// short spectra, and as two pairs of eight warps that read each template factor
+// once per pair 109.0 against 106.4 ms at 2^21 bins and 9.38 against 9.28 ms.
 #include <type_traits>
 
 #include "device_sync.cuh"

@@ -278,10 +278,9 @@ cudaError_t launch_normalise(const float2 *in, float2 *out, int64_t n, int B, cu
 // Consumers sum their cells of each row in fixed h order (FP32), keep
 // (max, argmax) per stage (lowest t on ties) and the statistics partials,
 // and release each slot per warp.  One launch serves every spectrum of a
-// batch (24 spectra of 2^13-2^16 bins: 727 -> 68 us); where a spectrum's cells
-// alone would leave SMs idle, its fundamentals are split over several blocks
-// (harm_ny) that meet in an atomic maximum (2^16 bins, 33 fundamentals: 31 ->
-// 14 us).  Every wait is bounded (about one
+// batch (24 spectra of 2^13-2^16 bins: 727 -> 68 us); a spectrum's fundamentals
+// are split over several blocks (harm_ny, chosen where the plan lays out its
+// launches) that meet in an atomic maximum (2^16 bins, 33 fundamentals: 31 -> 14 us).  Every wait is bounded (about one
 // second); on expiry the block sets the error flag and leaves after its
 // copies in flight have landed.
 // ---------------------------------------------------------------------------

@@ -260,9 +260,14 @@ int64_t transforms_for(const jerk_plan_s *pl, int64_t n) {
 }
 
 // Harmonic blocks of a spectrum of n bins: blocks of cells, times parts of its
-// nf fundamentals where the cells alone would leave SMs without a block (a part
-// keeps at least 8 fundamentals).  The split depends on the spectrum alone, so
-// its statistics are added in the same order in every batch.
+// nf fundamentals.  Two blocks run per SM at a time, a block costs its
+// fundamentals plus about kBlock of them for filling its ring and writing its
+// maxima, and whole waves count: the split is the one with the fewest steps
+// (300 007 bins: 147 blocks left every SM half empty, 549 -> 334 us; 700 001 bins:
+// 342 blocks were a second wave for 38 of them, 1174 -> 829 us; 2^21 bins, 1024
+// blocks: 10.95 -> 10.10 ms).  It depends on the spectrum alone, so its
+// statistics are added in the same order in every batch.
+constexpr int kMaxParts = 16;
 int64_t harm_nx_for(const jerk_plan_s *pl, int64_t n) {
     if (pl->prm.n_stages < 2) return 0;
     const int64_t cpb = harmonic_cells_per_block();
@@ -270,8 +275,18 @@ int64_t harm_nx_for(const jerk_plan_s *pl, int64_t n) {
 }
 
 int harm_ny_for(const jerk_plan_s *pl, int64_t nx, int nf) {
-    if (nx < 1) return 1;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(pl->sms / nx, nf / 8));
+    constexpr int kBlock = 6;
+    const int64_t slots = 2 * (int64_t)pl->sms;
+    int best = 1;
+    int64_t best_cost = INT64_MAX;
+    for (int ny = 1; ny <= kMaxParts && (ny == 1 || nf / ny >= 8); ++ny) {
+        const int64_t cost = (nx * ny + slots - 1) / slots * ((nf + ny - 1) / ny + kBlock);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = ny;
+        }
+    }
+    return best;
 }
 
 jerk_status validate(const jerk_params *p) {
@@ -902,9 +917,7 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
     pl->slot_cap = item_rows(pl, N, params->zmax, params->wmax, 0, nullptr, nullptr, nullptr, nullptr, nullptr) +
                    (int64_t)pl->max_batch * 32 * std::max(1, pl->n_fund * JERK_MAX_HARMONIC);
     const int64_t conv_blocks = (ctas_for(pl, N) + (int64_t)pl->max_batch * (int64_t)pl->groups.size()) * max_parts(pl);
-    // (a spectrum's harmonic blocks are at most one per SM more than its blocks of cells)
-    const int64_t harm_blocks = harm_nx_for(pl, N) + (int64_t)pl->max_batch *
-                                (1 + std::min<int64_t>(pl->sms, (int64_t)(pl->n_fund / 8 + 1) * (harm_nx_for(pl, N) + 1)));
+    const int64_t harm_blocks = kMaxParts * (harm_nx_for(pl, N) + (int64_t)pl->max_batch);
     // (a partial search by template range runs each group's templates of the range
     // and, separately, the other templates its fundamentals need: up to twice the CTAs)
     pl->stat_part_cap = 2 * 2 * conv_blocks + 2 * (int64_t)ns * harm_blocks;
