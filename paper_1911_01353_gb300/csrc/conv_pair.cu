@@ -4,33 +4,38 @@
 // One CTA holds three segments, four warps each, and walks a group of
 // templates.  A thread keeps 16 points of the even-cell and 16 of the odd-cell
 // half transform (2048 points each) side by side (pair.cuh), so its FP32 work
-// is packed: 2048 = 8 x 16 x 16, three passes in registers with one exchange
-// over the segment's 128 threads and one within 16 lanes, 16 bytes (a pair of
-// complex values) per shared-memory access.  Shared memory (32 KB per
-// exchange buffer) is swizzled, not padded: element i sits at i ^ ((i >> 4) & 7),
-// free of bank conflicts in every pass, and three buffers, the two-deep template
-// ring, three staged rows and 8-bit argmaxima fill 220 KB.  A thread's 160
-// tensor-memory columns hold what is the same for every template: the twiddles
-// (pass 0: a pair of factors per output, the even half's w_2048^{f r} and the
-// odd half's w_4096^{f (2r+1)}; pass 1: w_256^{f r}, each part twice, ready for
-// packed products) and the segment's spectrum, read 32 columns at a time.
+// is packed: 2048 = 8 x 16 x 16, three passes in registers.  The exchange after
+// pass 0 goes over the segment's 128 threads through shared memory, 16 bytes (a
+// pair of complex values) per access; the one after pass 1 stays within a warp
+// and goes through tensor memory (exchange16).  The exchange buffers (32 KB each)
+// are swizzled, not padded: element i sits at i ^ ((i >> 4) & 7) ^ ((i >> 6) & 4),
+// free of bank conflicts; three of them, the two-deep template ring, three staged
+// rows and 8-bit argmaxima fill 220 KB.  Tensor memory also holds what is the same
+// for every template: the twiddles (pass 0: a pair of factors per output, the even
+// half's w_2048^{f r} and the odd half's w_4096^{f (2r+1)}; pass 1: w_256^{f r},
+// each part twice, ready for packed products) and the segment's spectrum.
 //
 // Why three segments of four warps: the passes of one segment wait on barriers
 // over its four warps only, one warp on each of the SM's four schedulers, and
 // the other two segments fill those waits; 168 registers a thread hold 16
-// pairs (64), 32 columns on their way and the running maxima (32) without a
-// spill.  What bounds it is shared memory: about 1.5 K wavefronts per transform
-// (exchanges 1024, template factors 256, argmaxima, staged rows and metadata)
-// and 0.2 K of global traffic on the same pipe, four fifths of a step's 6.5 K
-// cycles for three transforms; FMA 55 % and issue 48 % (28 % fewer instructions
-// than with one complex value per register pair and 256 threads per segment).
-// Filter alone, bank of 12 261 templates, 2^21 bins, stages 1-2-4-8: 118.6 ->
-// 106.4 ms; 3131 templates, 700 001 bins: 10.37 -> 9.08 ms; six requests on the
-// bank of 27 391 templates, stage 1: 10.75 -> 9.28 ms.  Four segments a CTA
-// were not faster: as four of four warps (maxima in tensor memory, pass-1
-// twiddles in shared memory, rows staged in the exchange buffer) 27 % slower on
-// short spectra, and as two pairs of eight warps that read each template factor
-// once per pair 109.0 against 106.4 ms at 2^21 bins and 9.38 against 9.28 ms.
+// pairs (64), factors on their way and the running maxima (32) without a
+// spill.  What bounds it is latency at these 12 warps: FMA 61 %, issue 54 %,
+// shared memory 50 % (about 1.0 K wavefronts per transform: exchange 512, template
+// factors 256, argmaxima, staged rows and metadata) of their peaks, none of them
+// full.  With both exchanges in shared memory (1.5 K wavefronts) that pipe was the
+// bound, at 71 %.  Filter alone, bank of 12 261 templates, 2^21 bins, stages
+// 1-2-4-8: 118.6 ms with one complex value per register pair and 256 threads per
+// segment, 106.4 ms as pairs, 103.3 ms with the second exchange in tensor memory;
+// 3131 templates, 700 001 bins: 10.37, 9.08, 8.83 ms; six requests on the bank of
+// 27 391 templates, stage 1: 10.75, 9.28, 9.19 ms.
+//
+// Not faster: the factors' loads issued a whole pass earlier (103.5 ms, and 104.2
+// with the spectrum's a template earlier), so their latency is hidden already.
+// Four segments a CTA, with both exchanges in shared memory: as four of four
+// warps (maxima in tensor memory, pass-1 twiddles in shared memory, rows staged in
+// the exchange buffer) 27 % slower on short spectra, and as two pairs of eight
+// warps that read each template factor once per pair 109.0 against 106.4 ms at
+// 2^21 bins and 9.38 against 9.28 ms.
 #include <type_traits>
 
 #include "device_sync.cuh"
@@ -50,7 +55,13 @@ constexpr int OFF_WORK = NBUF * L * 8;
 constexpr int OFF_STAGE = OFF_WORK + SEGS * WORKB;        // staged power row, float [L] per segment
 constexpr int OFF_AMX = OFF_STAGE + SEGS * L * 4;         // argmax within kFlush templates, uint8 [32][NT] per segment
 constexpr int SMEM = OFF_AMX + SEGS * L;
-constexpr uint32_t TMCOLS = 512, TMSLOT = 160;            // tensor-memory columns: allocated, per thread
+// tensor-memory columns: twiddles 0 .. 123 (the same words for the three segments'
+// warps of a lane range), then 128 per segment: spectrum 32, statistics 4, exchange 64
+constexpr uint32_t TMCOLS = 512, TMSEG = 128, TMSTAT = 32, TMX = 64;
+
+// Pass 1's twiddled outputs in the order in which the exchange sends them (and
+// their factors lie in tensor memory): 4, 8, 12, then 1, 5, 9, 13, and so on.
+__host__ __device__ constexpr int order1(int q) { return (4 * (q + 1)) % 16 + (q + 1) / 4; }
 
 // The forward transform's twiddles: the conjugates of the inverse's even-half
 // factors, from this thread's tensor-memory columns.
@@ -76,7 +87,7 @@ struct FftTwFwd {
             tmem_wait_ld32(x);
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (8 * c + q + 1 < 16) a[8 * c + q + 1] = cmul(a[8 * c + q + 1], w(x, q));
+                if (8 * c + q < 15) a[order1(8 * c + q)] = cmul(a[order1(8 * c + q)], w(x, q));
         }
     }
 };
@@ -94,9 +105,64 @@ __device__ __forceinline__ void sts_pair(uint32_t addr, cpair v) {
 }
 
 // times the q-th twiddle pair of 32 tensor-memory columns: (re, re, im, im) each
-__device__ __forceinline__ cpair mul_tw(cpair a, const uint32_t (&w)[32], int q) {
+template <int N>
+__device__ __forceinline__ cpair mul_tw(cpair a, const uint32_t (&w)[N], int q) {
     return mul(a, make_float2(__uint_as_float(w[4 * q]), __uint_as_float(w[4 * q + 1])),
                make_float2(__uint_as_float(w[4 * q + 2]), __uint_as_float(w[4 * q + 3])));
+}
+
+__device__ __forceinline__ uint32_t word(const cpair &v, int w) {
+    return __float_as_uint(w == 0 ? v.re.x : w == 1 ? v.re.y : w == 2 ? v.im.x : v.im.y);
+}
+// The exchange between passes 1 and 2 through tensor memory.  Thread 2 i + s of
+// the warp holds v[r], r = 0 .. 15, of point i of sub-problem s; thread 16 s + r
+// leaves with v[i], i = 0 .. 15.  A store of 64 columns by lane and a load of 16
+// lanes x 64 columns moves two bits of the register index into the low bits of
+// the lane index and the lane index's two high bits into the registers: twice
+// that is the whole transpose.
+//
+// First store, 16 columns of it: outputs r = t, t + 4, t + 8, t + 12
+__device__ __forceinline__ void send16(const cpair (&v)[16], uint32_t tx, int t) {
+    uint32_t x[16];
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int w = 0; w < 4; ++w) x[8 * (w >> 1) + 2 * b + (w & 1)] = word(v[t + 4 * b], w);
+    tmem_st16(tx + 16 * t, x);
+}
+// the rest of it
+__device__ __forceinline__ void exchange16(cpair (&v)[16], uint32_t tx) {
+    uint32_t y[4][16];                                        // [2 h + u]: lanes 16 h .., columns 32 u ..
+    tmem_wait_st();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) tmem_ld16x32(tx + ((16u * (e >> 1)) << 16) + 32 * (e & 1), y[e]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) tmem_wait_ld16(y[e]);
+    // y[2 h + u][4 q + 2 k + p]: point 8 h + 4 k + (lane >> 3), sub-problem (lane >> 2) & 1,
+    // r = 4 (lane & 3) + 2 u + (q >> 1), word 2 (q & 1) + p
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {                             // t = 2 h + k
+        uint32_t x[16];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+                x[8 * (q & 1) + 2 * (q >> 1) + p] = y[(t & 2) + (q >> 2)][4 * (q & 3) + 2 * (t & 1) + p];
+        tmem_st16(tx + 16 * t, x);
+    }
+    tmem_wait_st();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) tmem_ld16x32(tx + ((16u * (e >> 1)) << 16) + 32 * (e & 1), y[e]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) tmem_wait_ld16(y[e]);
+    // y[2 H + u][4 Q + 2 K + p]: point 8 u + 4 (Q >> 1) + 2 H + K, word 2 (Q & 1) + p
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const uint32_t(&z)[16] = y[(i & 2) + (i >> 3)];
+        const int o = 4 * (2 * ((i >> 2) & 1)) + 2 * (i & 1);
+        v[i].re = make_float2(__uint_as_float(z[o]), __uint_as_float(z[o + 1]));
+        v[i].im = make_float2(__uint_as_float(z[o + 4]), __uint_as_float(z[o + 5]));
+    }
 }
 
 template <bool ROWS>
@@ -180,37 +246,39 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
                       &full[b]);
         }
 
-    // ---- twiddles into this thread's tensor-memory columns ---------------------
+    // ---- twiddles into tensor memory ---------------------------------------------
     // column 4 c, c = 8 i + r: pass 0, item i (f = j + 128 i), output r: even-half and
-    // odd-half factors (re, re, im, im); c = 15 + r: pass 1, output r, each part twice
-    const uint32_t tcol = tslot + ((uint32_t)(32 * (warp & 3)) << 16) + TMSLOT * (uint32_t)(warp >> 2);
-    // (the three segments need the same: each computes a third, into the exchange buffers)
-    float *tws = reinterpret_cast<float *>(sm + OFF_WORK) + j;                 // word w of thread j at [w][j]
+    // odd-half factors (re, re, im, im); c = 16 + q: pass 1, output order1(q), each part twice
+    const uint32_t tcol = tslot + ((uint32_t)(32 * (warp & 3)) << 16);
+    const uint32_t tseg = tcol + TMSEG * (uint32_t)(1 + seg);
+    // pass 1 works on sub-problem jj >> 4, point jj & 15 (see the exchange below)
+    const int jj = (j & 96) + 16 * (j & 1) + ((j & 31) >> 1);
+    // (the three segments' warps of a lane range compute a third each)
 #pragma unroll 1
-    for (int c = seg; c < 32; c += SEGS) {
-        float2 wx, wy;
-        if (c < 16) {
-            const int f = j + NT * (c >> 3), r = c & 7;
-            wx = unit_root<+1>((2 * f * r) & (L - 1), L);
-            wy = unit_root<+1>((f * (2 * r + 1)) & (L - 1), L);
-        } else {
-            wx = wy = unit_root<+1>(((j & 15) * (c - 15)) & 255, 256);
-        }
-        tws[NT * (4 * c)] = wx.x;
-        tws[NT * (4 * c + 1)] = wy.x;
-        tws[NT * (4 * c + 2)] = wx.y;
-        tws[NT * (4 * c + 3)] = wy.y;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
+    for (int c = seg; c < 16; c += SEGS) {
         float x[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) x[q] = tws[NT * (8 * c + q)];
+        for (int u = 0; u < 2; ++u) {
+            const int d = 2 * c + u;
+            float2 wx, wy;
+            if (d < 16) {
+                const int f = j + NT * (d >> 3), r = d & 7;
+                wx = unit_root<+1>((2 * f * r) & (L - 1), L);
+                wy = unit_root<+1>((f * (2 * r + 1)) & (L - 1), L);
+            } else {
+                wx = wy = unit_root<+1>(((jj & 15) * (d == 31 ? 0 : order1(d - 16))) & 255, 256);
+            }
+            x[4 * u] = wx.x;
+            x[4 * u + 1] = wy.x;
+            x[4 * u + 2] = wx.y;
+            x[4 * u + 3] = wy.y;
+        }
         tmem_st8(tcol + 8 * c, x);
     }
-    __syncthreads();
     tmem_wait_st();
+    tmem_fence_before();
+    __syncthreads();
+    tmem_fence_after();
 
     // ---- 1. forward transform of the segment's bins (2048 points) ----------------
     // this thread keeps the spectrum values it multiplies: X[j + 128 m] (the
@@ -228,8 +296,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
         }
         fft_pass0<11, -1>(v, twf);
         fft_store0<11>(v, work, j);
-        fft_rest<11, -1>(v, work, j, twf, bar_seg);
-        const int rf = fft_rev<11>(j);
+        fft_rest<11, -1>(v, work, jj, twf, bar_seg);
+        const int rf = fft_rev<11>(jj);
         bar_seg();                                            // all reads of `work` done
 #pragma unroll
         for (int r = 0; r < 16; ++r) work[rf + NT * r] = v[r];
@@ -243,7 +311,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
                 x[2 * q] = t.x;
                 x[2 * q + 1] = t.y;
             }
-            tmem_st8(tcol + 128 + 8 * c, x);
+            tmem_st8(tseg + 8 * c, x);
         }
         tmem_wait_st();
     }
@@ -251,8 +319,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     // ---- 2. templates of this group -----------------------------------------
     const uint32_t wb = smem_u32(work);
     const uint32_t w0 = wb + 16u * (uint32_t)(j ^ ((j >> 4) & 7));                       // pass-0 stores
-    const uint32_t w1 = wb + 16u * (uint32_t)((j >> 4) * 256 + (j & 15));                // pass 1
-    const uint32_t w2 = wb + 16u * (uint32_t)(16 * j + (j & 7));                         // pass-2 loads
+    const uint32_t w1 = wb + 16u * (uint32_t)((jj >> 4) * 256 + ((jj & 15) ^ (4 * (j & 1))));   // pass-1 loads
     // this thread's outputs: cells c0 + 256 r + (0, 1)
     const int c0 = 2 * (j >> 4) + 16 * (j & 15);
     unsigned vmask = 0;
@@ -276,13 +343,13 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     // their FP64 sums sit in the last four of this thread's tensor-memory columns
     auto add_stats = [&] {
         double d0, d1;
-        tmem_ld_f64x2(tcol + 124, d0, d1);
+        tmem_ld_f64x2(tseg + TMSTAT, d0, d1);
         d0 += (double)fa0;
         d1 += (double)fa1;
-        tmem_st_f64x2(tcol + 124, d0, d1);
+        tmem_st_f64x2(tseg + TMSTAT, d0, d1);
         fa0 = fa1 = 0.f;
     };
-    if constexpr (STATS) tmem_st_f64x2(tcol + 124, 0.0, 0.0);
+    if constexpr (STATS) tmem_st_f64x2(tseg + TMSTAT, 0.0, 0.0);
     // Running maxima of the templates tb + base .. into the stage-1
     // max-projection, through the exchange buffer so that a warp's atomics fall on
     // 32 consecutive cells (straight from the registers each lane's was a sector of
@@ -327,7 +394,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
             const int it = k - tb;
             const int b = it % NBUF;
             uint32_t x[32];
-            tmem_ld32(tcol + 128, x);
+            tmem_ld32(tseg, x);
             // A thread whose wait expired reads a buffer that may still be landing;
             // its values are discarded: the whole segment leaves at the barrier below.
             const bool ok = mbar_wait_bounded(&full[b], (uint32_t)(it / NBUF) & 1u);
@@ -366,7 +433,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int r = 0; r < 8; ++r) sts_pair(w0 + 16 * (256 * r + NT * i), v[2 * r + i]);
+                for (int r = 0; r < 8; ++r) sts_pair((w0 ^ (64u * (r & 1))) + 16 * (256 * r + NT * i), v[2 * r + i]);
             // the segment's last warp releases (and, last of the segments, refills) the buffer
             if (j == NT - 32) __threadfence_block();
             if (j == NT - 32 && atomicAdd(&rel[b], 1) == SEGS - 1) {
@@ -412,7 +479,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
                     store_rows(a, rent[seg][(k - 1) & 1], mp.e1 - mp.e0, stage, sbound[seg], seg0, j, NT, kChkRowStore);
             }
             bar_seg();
-            // pass 1: sub-problem j / 16, points (j & 15) + 16 k
+            // pass 1: sub-problem jj / 16, points (jj & 15) + 16 k
 #pragma unroll
             for (int k1 = 0; k1 < 4; ++k1)
 #pragma unroll
@@ -420,30 +487,29 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
                     const int m = k1 + 4 * k2;
                     v[m] = lds_pair((w1 ^ (16u * (m & 7))) + 256 * m);
                 }
+            uint32_t xa[16], xb[16];
+            tmem_ld16(tcol + 64, xa);
             dft16(v);
-            tmem_ld32(tcol + 64, x);
-            tmem_wait_ld32(x);
+            tmem_wait_ld16(xa);
+            tmem_ld16(tcol + 80, xb);
 #pragma unroll
-            for (int r = 1; r < 9; ++r) v[r] = mul_tw(v[r], x, r - 1);
-            tmem_ld32(tcol + 96, x);
-            // exchange within the 16 threads of the sub-problem (one half of a warp)
-            __syncwarp();
+            for (int q = 0; q < 4; ++q) v[order1(q)] = mul_tw(v[order1(q)], xa, q);
+            send16(v, tseg + TMX, 0);
+            tmem_wait_ld16(xb);
+            tmem_ld16(tcol + 96, xa);
 #pragma unroll
-            for (int r = 0; r < 9; ++r) sts_pair((w1 ^ (16u * (r & 7))) + 256 * r, v[r]);
-            tmem_wait_ld32(x);
+            for (int q = 4; q < 8; ++q) v[order1(q)] = mul_tw(v[order1(q)], xb, q - 4);
+            send16(v, tseg + TMX, 1);
+            tmem_wait_ld16(xa);
+            tmem_ld16(tcol + 112, xb);
 #pragma unroll
-            for (int r = 9; r < 16; ++r) {
-                v[r] = mul_tw(v[r], x, r - 9);
-                sts_pair((w1 ^ (16u * (r & 7))) + 256 * r, v[r]);
-            }
-            __syncwarp();
+            for (int q = 8; q < 12; ++q) v[order1(q)] = mul_tw(v[order1(q)], xa, q - 8);
+            send16(v, tseg + TMX, 2);
+            tmem_wait_ld16(xb);
 #pragma unroll
-            for (int k1 = 0; k1 < 4; ++k1)
-#pragma unroll
-                for (int k2 = 0; k2 < 4; ++k2) {
-                    const int m = k1 + 4 * k2;
-                    v[m] = lds_pair((w2 ^ (16u * (m & 7))) + 16 * (m & 8));
-                }
+            for (int q = 12; q < 15; ++q) v[order1(q)] = mul_tw(v[order1(q)], xb, q - 12);
+            send16(v, tseg + TMX, 3);
+            exchange16(v, tseg + TMX);
             dft16(v);
             float2 P[16];
 #pragma unroll
@@ -525,7 +591,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     double d0 = 0.0, d1 = 0.0;
     if constexpr (STATS) {
         add_stats();
-        tmem_ld_f64x2(tcol + 124, d0, d1);
+        tmem_ld_f64x2(tseg + TMSTAT, d0, d1);
     }
     tmem_fence_before();
     __syncthreads();

@@ -33,12 +33,8 @@ __device__ __forceinline__ cpair mul(cpair a, float2 wr, float2 wi) {
 __device__ __forceinline__ cpair mulc(cpair a, float c, float s) {
     return {fma2k(-s, a.im, mul2(a.re, make_float2(c, c))), fma2k(s, a.re, mul2(a.im, make_float2(c, c)))};
 }
-// (u, v) with exp(2 pi i / 8) b = (u + i v) / sqrt 2, and the same for exp(6 pi i / 8)
+// (u, v) with exp(2 pi i / 8) b = (u + i v) / sqrt 2
 __device__ __forceinline__ cpair eighth1(cpair b) { return {sub2(b.re, b.im), add2(b.im, b.re)}; }
-__device__ __forceinline__ cpair eighth3(cpair b) {
-    const float2 s = add2(b.re, b.im);
-    return {make_float2(-s.x, -s.y), sub2(b.re, b.im)};
-}
 
 __device__ __forceinline__ void dft4(cpair &a0, cpair &a1, cpair &a2, cpair &a3) {
     const cpair s02 = a0 + a2, d02 = a0 - a2, s13 = a1 + a3, e13 = a1 - a3;
@@ -62,7 +58,7 @@ __device__ __forceinline__ void dft8(cpair &a0, cpair &a1, cpair &a2, cpair &a3,
     a5 = axpy(-kRsqrt2, q1, c1);
     a2 = add_i(c2, o2);
     a6 = sub_i(c2, o2);
-    const cpair s = {add2(o3.re, o3.im), sub2(o3.im, o3.re)};  // -eighth3(o3)
+    const cpair s = {add2(o3.re, o3.im), sub2(o3.im, o3.re)};  // -(u, v) of exp(6 pi i / 8) o3
     a3 = axpy(-kRsqrt2, s, c3);
     a7 = axpy(kRsqrt2, s, c3);
 }
@@ -102,7 +98,7 @@ __device__ __forceinline__ void dft16(cpair (&a)[16]) {
         y[14] = {fma2k(kRsqrt2, qf.im, d02.re), fma2k(-kRsqrt2, qf.re, d02.im)};
     }
     {
-        const cpair s = {add2(a[14].re, a[14].im), sub2(a[14].im, a[14].re)};   // -eighth3(a[14])
+        const cpair s = {add2(a[14].re, a[14].im), sub2(a[14].im, a[14].re)};   // -(u, v) of exp(6 pi i / 8) a[14]
         const cpair s02 = axpy(-kRsqrt2, s, a[12]), d02 = axpy(kRsqrt2, s, a[12]);
         const cpair x1 = mulc(a[13], S1, C1), x3 = mulc(a[15], -C1, -S1);
         const cpair s13 = x1 + x3, e13 = x1 - x3;
