@@ -7,27 +7,35 @@
 // is packed: 2048 = 8 x 16 x 16, three passes in registers.  The exchange after
 // pass 0 goes over the segment's 128 threads through shared memory, 16 bytes (a
 // pair of complex values) per access; the one after pass 1 stays within a warp
-// and goes through tensor memory (exchange16).  The exchange buffers (32 KB each)
-// are swizzled, not padded: element i sits at i ^ ((i >> 4) & 7) ^ ((i >> 6) & 4),
-// free of bank conflicts; three of them, the two-deep template ring, three staged
-// rows and 8-bit argmaxima fill 220 KB.  Tensor memory also holds what is the same
-// for every template: the twiddles (pass 0: a pair of factors per output, the even
-// half's w_2048^{f r} and the odd half's w_4096^{f (2r+1)}; pass 1: w_256^{f r},
-// each part twice, ready for packed products) and the segment's spectrum.
+// and goes through tensor memory (exchange16).  The exchange buffers are padded
+// (element i of sub-problem r at 276 r + i + i / 16), so that every access is free
+// of bank conflicts and an immediate away from one base; three of them, the
+// two-deep template ring and three staged rows fill 216 KB.  Tensor memory also
+// holds what is the same for every template: the twiddles (pass 0: a pair of
+// factors per output, the even half's w_2048^{f r} and the odd half's
+// w_4096^{f (2r+1)}; pass 1: w_256^{f r}, each part twice, ready for packed
+// products) and the segment's spectrum.  Its addresses are broadcast from lane 0
+// once, so that the compiler keeps them in uniform registers.
 //
 // Why three segments of four warps: the passes of one segment wait on barriers
 // over its four warps only, one warp on each of the SM's four schedulers, and
 // the other two segments fill those waits; 168 registers a thread hold 16
-// pairs (64), factors on their way and the running maxima (32) without a
-// spill.  What bounds it is latency at these 12 warps: FMA 61 %, issue 54 %,
-// shared memory 50 % (about 1.0 K wavefronts per transform: exchange 512, template
-// factors 256, argmaxima, staged rows and metadata) of their peaks, none of them
-// full.  With both exchanges in shared memory (1.5 K wavefronts) that pipe was the
-// bound, at 71 %.  Filter alone, bank of 12 261 templates, 2^21 bins, stages
-// 1-2-4-8: 118.6 ms with one complex value per register pair and 256 threads per
-// segment, 106.4 ms as pairs, 103.3 ms with the second exchange in tensor memory;
-// 3131 templates, 700 001 bins: 10.37, 9.08, 8.83 ms; six requests on the bank of
-// 27 391 templates, stage 1: 10.75, 9.28, 9.19 ms.
+// pairs (64), factors on their way, the running maxima (32) and their 8-bit
+// argmaxima (8) without a spill.  What bounds it is latency at these 12 warps:
+// FMA 61 %, issue 54 %, shared memory 46 % of their peaks, none of them full
+// (with both exchanges in shared memory that pipe was the bound, at 71 %).  Filter alone, ms:
+//
+//                                         12 261 templates,  3131 templates,  27 391 templates,
+//                                         2^21 bins, stages  700 001 bins     six requests,
+//                                         1-2-4-8                             stage 1
+//   one complex value per register pair,
+//   256 threads a segment                 118.6              10.37            10.75
+//   pairs, 128 threads a segment          106.4               9.08             9.28
+//   second exchange in tensor memory      103.3               8.83             9.19
+//   its second store 2 columns at a time,
+//   uniform addresses                     101.1               8.65             9.14
+//   argmaxima in registers                101.2               8.66             8.96
+//   first exchange padded, not swizzled   100.1               8.58             8.84
 //
 // Not faster: the factors' loads issued a whole pass earlier (103.5 ms, and 104.2
 // with the spectrum's a template earlier), so their latency is hidden already.
@@ -48,13 +56,13 @@
 namespace jerk {
 namespace {
 
-constexpr int L = 4096, HALF = L / 2, NT = 128, SEGS = kPairSegs, THREADS = SEGS * NT, NBUF = 2;
+constexpr int L = 4096, NT = 128, SEGS = kPairSegs, THREADS = SEGS * NT, NBUF = 2;
 constexpr int kFlush = 256;                               // templates per 8-bit argmax
-constexpr int WORKB = HALF * 16;                          // exchange buffer of a segment (bytes)
+constexpr int PADSUB = 256 + 16 + 4;                      // a sub-problem of 256 pairs, padded: i + i / 16, and 4 apart
+constexpr int WORKB = 8 * PADSUB * 16;                    // exchange buffer of a segment (bytes)
 constexpr int OFF_WORK = NBUF * L * 8;
 constexpr int OFF_STAGE = OFF_WORK + SEGS * WORKB;        // staged power row, float [L] per segment
-constexpr int OFF_AMX = OFF_STAGE + SEGS * L * 4;         // argmax within kFlush templates, uint8 [32][NT] per segment
-constexpr int SMEM = OFF_AMX + SEGS * L;
+constexpr int SMEM = OFF_STAGE + SEGS * L * 4;
 // tensor-memory columns: twiddles 0 .. 123 (the same words for the three segments'
 // warps of a lane range), then 128 per segment: spectrum 32, statistics 4, exchange 64
 constexpr uint32_t TMCOLS = 512, TMSEG = 128, TMSTAT = 32, TMX = 64;
@@ -130,7 +138,8 @@ __device__ __forceinline__ void send16(const cpair (&v)[16], uint32_t tx, int t)
         for (int w = 0; w < 4; ++w) x[8 * (w >> 1) + 2 * b + (w & 1)] = word(v[t + 4 * b], w);
     tmem_st16(tx + 16 * t, x);
 }
-// the rest of it
+// the rest of it (its store two columns at a time: the loads leave pairs that are
+// two apart, and 16-column stores took 64 register moves to gather them)
 __device__ __forceinline__ void exchange16(cpair (&v)[16], uint32_t tx) {
     uint32_t y[4][16];                                        // [2 h + u]: lanes 16 h .., columns 32 u ..
     tmem_wait_st();
@@ -141,15 +150,11 @@ __device__ __forceinline__ void exchange16(cpair (&v)[16], uint32_t tx) {
     // y[2 h + u][4 q + 2 k + p]: point 8 h + 4 k + (lane >> 3), sub-problem (lane >> 2) & 1,
     // r = 4 (lane & 3) + 2 u + (q >> 1), word 2 (q & 1) + p
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {                             // t = 2 h + k
-        uint32_t x[16];
+    for (int t = 0; t < 4; ++t)                               // t = 2 h + k
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-#pragma unroll
-            for (int p = 0; p < 2; ++p)
-                x[8 * (q & 1) + 2 * (q >> 1) + p] = y[(t & 2) + (q >> 2)][4 * (q & 3) + 2 * (t & 1) + p];
-        tmem_st16(tx + 16 * t, x);
-    }
+            tmem_st2(tx + 16 * t + 8 * (q & 1) + 2 * (q >> 1), y[(t & 2) + (q >> 2)][4 * (q & 3) + 2 * (t & 1)],
+                     y[(t & 2) + (q >> 2)][4 * (q & 3) + 2 * (t & 1) + 1]);
     tmem_wait_st();
 #pragma unroll
     for (int e = 0; e < 4; ++e) tmem_ld16x32(tx + ((16u * (e >> 1)) << 16) + 32 * (e & 1), y[e]);
@@ -164,6 +169,9 @@ __device__ __forceinline__ void exchange16(cpair (&v)[16], uint32_t tx) {
         v[i].im = make_float2(__uint_as_float(z[o + 4]), __uint_as_float(z[o + 5]));
     }
 }
+
+// byte_perm selector: byte b from the second operand's lowest
+__host__ __device__ constexpr uint32_t sel_byte(int b) { return 0x3210u ^ ((uint32_t)(b ^ 4) << (4 * b)); }
 
 template <bool ROWS>
 __device__ __forceinline__ int bank_row(const ConvArgs &a, int k) {
@@ -190,7 +198,6 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     float2 *ring = reinterpret_cast<float2 *>(sm);
     float2 *work = reinterpret_cast<float2 *>(sm + OFF_WORK + seg * WORKB);
     float *stage = reinterpret_cast<float *>(sm + OFF_STAGE) + seg * L;
-    uint8_t *amx = sm + OFF_AMX + seg * L + j;                // + NT * (2 r + lane)
     const SyncNamed bar_seg{1 + seg, NT};
 
     // (spectrum, template group) entry of this CTA
@@ -249,8 +256,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     // ---- twiddles into tensor memory ---------------------------------------------
     // column 4 c, c = 8 i + r: pass 0, item i (f = j + 128 i), output r: even-half and
     // odd-half factors (re, re, im, im); c = 16 + q: pass 1, output order1(q), each part twice
-    const uint32_t tcol = tslot + ((uint32_t)(32 * (warp & 3)) << 16);
-    const uint32_t tseg = tcol + TMSEG * (uint32_t)(1 + seg);
+    const uint32_t tcol = __shfl_sync(0xffffffffu, tslot + ((uint32_t)(32 * (warp & 3)) << 16), 0);
+    const uint32_t tseg = __shfl_sync(0xffffffffu, tcol + TMSEG * (uint32_t)(1 + seg), 0);
     // pass 1 works on sub-problem jj >> 4, point jj & 15 (see the exchange below)
     const int jj = (j & 96) + 16 * (j & 1) + ((j & 31) >> 1);
     // (the three segments' warps of a lane range compute a third each)
@@ -318,8 +325,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
 
     // ---- 2. templates of this group -----------------------------------------
     const uint32_t wb = smem_u32(work);
-    const uint32_t w0 = wb + 16u * (uint32_t)(j ^ ((j >> 4) & 7));                       // pass-0 stores
-    const uint32_t w1 = wb + 16u * (uint32_t)((jj >> 4) * 256 + ((jj & 15) ^ (4 * (j & 1))));   // pass-1 loads
+    const uint32_t w0 = wb + 16u * (uint32_t)(j + (j >> 4));                             // pass-0 stores
+    const uint32_t w1 = wb + 16u * (uint32_t)((jj >> 4) * PADSUB + (jj & 15));           // pass-1 loads
     // this thread's outputs: cells c0 + 256 r + (0, 1)
     const int c0 = 2 * (j >> 4) + 16 * (j & 15);
     unsigned vmask = 0;
@@ -336,6 +343,9 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
         }
         if (V >= 256 * RSAFE && seg0w + 256 * RSAFE <= bN) vmask |= 1u << 16;
     }
+    uint32_t am[8];                                           // argmax bytes: position within kFlush templates
+#pragma unroll
+    for (int q = 0; q < 8; ++q) am[q] = 0;
     float2 mx[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) mx[r] = make_float2(-1.0f, -1.0f);
@@ -365,7 +375,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
 #pragma unroll
             for (int l = 0; l < 2; ++l) {
                 // (a cell that is not a number under every template has no argmax: any valid position)
-                const int t = __ldg(a.order + min(tb + base + (int)amx[NT * (2 * r + l)], te - 1));
+                const int t = __ldg(a.order + min(tb + base + (int)((am[(2 * r + l) >> 2] >> (8 * ((2 * r + l) & 3))) & 255u), te - 1));
                 v[l] = ((unsigned long long)__float_as_uint(l ? mx[r].y : mx[r].x) << 32) |
                        (unsigned long long)(0xFFFFFFFFu - (unsigned)t);
             }
@@ -433,7 +443,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int r = 0; r < 8; ++r) sts_pair((w0 ^ (64u * (r & 1))) + 16 * (256 * r + NT * i), v[2 * r + i]);
+                for (int r = 0; r < 8; ++r) sts_pair(w0 + 16 * (PADSUB * r + (NT + NT / 16) * i), v[2 * r + i]);
             // the segment's last warp releases (and, last of the segments, refills) the buffer
             if (j == NT - 32) __threadfence_block();
             if (j == NT - 32 && atomicAdd(&rel[b], 1) == SEGS - 1) {
@@ -485,7 +495,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
 #pragma unroll
                 for (int k2 = 0; k2 < 4; ++k2) {
                     const int m = k1 + 4 * k2;
-                    v[m] = lds_pair((w1 ^ (16u * (m & 7))) + 256 * m);
+                    v[m] = lds_pair(w1 + 16 * 17 * m);
                 }
             uint32_t xa[16], xb[16];
             tmem_ld16(tcol + 64, xa);
@@ -521,11 +531,11 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
                 for (int r = 0; r < RK; ++r) {
                     if (P[r].x > mx[r].x) {
                         mx[r].x = P[r].x;
-                        amx[NT * (2 * r)] = (uint8_t)it;      // rare after the first templates
+                        am[(2 * r) >> 2] = __byte_perm(am[(2 * r) >> 2], it, sel_byte((2 * r) & 3));
                     }
                     if (P[r].y > mx[r].y) {
                         mx[r].y = P[r].y;
-                        amx[NT * (2 * r + 1)] = (uint8_t)it;
+                        am[(2 * r + 1) >> 2] = __byte_perm(am[(2 * r + 1) >> 2], it, sel_byte((2 * r + 1) & 3));
                     }
                 }
                 // harmonic rows of this template: stage the power row now, store it

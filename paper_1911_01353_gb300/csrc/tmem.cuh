@@ -85,6 +85,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&x)[16
                  : "memory");
 }
 
+// start loading 16 consecutive columns of this thread's lane (waited for by tmem_wait_ld16)
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, "
                  "%8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -93,6 +94,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
                    "=r"(r[15])
                  : "r"(taddr)
                  : "memory");
+}
+
+// 2 consecutive columns of this thread's lane (warp-collective)
+__device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t a, uint32_t b) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(a), "r"(b) : "memory");
 }
 
 // Start loading 32 columns of 16 lanes (taddr's, a multiple of 16, and the next
