@@ -20,8 +20,8 @@ namespace jerk {
 // cannot decide the rounding, so that the result is the FP64 one bit for bit.
 // FP64 instructions run at 1/64 of the FP32 rate, and sorting all FP64 powers
 // (55 barriers), then keying and scaling all bins in FP64, were the longest
-// parts: 2^16 bins 24 -> 9 us, 2^21 bins 170 -> 89 -> 76 us, a batch of 24
-// spectra of 2^13-2^16 bins 555 -> 40 -> 34 us.  Blocks that are too small or too large for FP32
+// parts: 2^16 bins 24 -> 10 us, 2^21 bins 170 -> 39 us, a batch of 24 spectra of
+// 2^13-2^16 bins 555 -> 34 us.  Blocks that are too small or too large for FP32
 // powers take the FP64 powers rounded to FP32, which keep the order.  One warp
 // per block of up to 1024 bins (four above, or where there are few blocks);
 // one launch normalises up to kNormItems spectra.
