@@ -29,7 +29,7 @@
 // registers for the 32 running maxima a thread has in this layout.  Bank of
 // 12 261 templates, 2^20 bins, FP16: filter 50.3 -> 44.7 ms, results unchanged
 // bit for bit.  The bound is still latency: shared memory (operands, template,
-// twiddles and the products' own reads) 55 %, issue 43 %, tensor pipe 31 %.
+// twiddles and the products' own reads) 57 %, issue 42 %, tensor pipe 25 %.
 //
 // Scaling: each segment spectrum is divided by max|X| * max|C| over the bank,
 // so |Z| <= 1 and the FP16 operands of both steps stay in range (|U'| <= 64,
