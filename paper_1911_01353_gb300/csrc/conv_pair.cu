@@ -36,6 +36,8 @@
 //   uniform addresses                     101.1               8.65             9.14
 //   argmaxima in registers                101.2               8.66             8.96
 //   first exchange padded, not swizzled   100.1               8.58             8.84
+//   loads and stores of the second
+//   exchange under one another             99.2               8.50             8.70
 //
 // Not faster: the factors' loads issued a whole pass earlier (103.5 ms, and 104.2
 // with the spectrum's a template earlier), so their latency is hidden already.
@@ -43,7 +45,9 @@
 // warps (maxima in tensor memory, pass-1 twiddles in shared memory, rows staged in
 // the exchange buffer) 27 % slower on short spectra, and as two pairs of eight
 // warps that read each template factor once per pair 109.0 against 106.4 ms at
-// 2^21 bins and 9.38 against 9.28 ms.
+// 2^21 bins and 9.38 against 9.28 ms.  One barrier per template, the buffers handed
+// back through mbarriers: 101.6 against 100.1 ms.  The second round's loads under its
+// stores as well: 100.8 against 99.2 ms.
 #include <type_traits>
 
 #include "device_sync.cuh"
@@ -138,13 +142,23 @@ __device__ __forceinline__ void send16(const cpair (&v)[16], uint32_t tx, int t)
         for (int w = 0; w < 4; ++w) x[8 * (w >> 1) + 2 * b + (w & 1)] = word(v[t + 4 * b], w);
     tmem_st16(tx + 16 * t, x);
 }
-// the rest of it (its store two columns at a time: the loads leave pairs that are
-// two apart, and 16-column stores took 64 register moves to gather them)
+// The rest of it, with t = 0, 1 sent, and the first stage of pass 2.  The first
+// round's loads of columns 0 .. 31 run under the stores of the others, the last
+// round's of the upper lanes under the butterflies of the lower ones.  The second
+// store goes two columns at a time: the loads leave pairs that are two apart, and
+// 16-column stores took 64 register moves to gather them.
 __device__ __forceinline__ void exchange16(cpair (&v)[16], uint32_t tx) {
     uint32_t y[4][16];                                        // [2 h + u]: lanes 16 h .., columns 32 u ..
-    tmem_wait_st();
 #pragma unroll
-    for (int e = 0; e < 4; ++e) tmem_ld16x32(tx + ((16u * (e >> 1)) << 16) + 32 * (e & 1), y[e]);
+    for (int u = 0; u < 2; ++u) {
+        if (u == 1) {
+            send16(v, tx, 2);
+            send16(v, tx, 3);
+        }
+        tmem_wait_st();
+        tmem_ld16x32(tx + 32 * u, y[u]);
+        tmem_ld16x32(tx + (16u << 16) + 32 * u, y[2 + u]);
+    }
 #pragma unroll
     for (int e = 0; e < 4; ++e) tmem_wait_ld16(y[e]);
     // y[2 h + u][4 q + 2 k + p]: point 8 h + 4 k + (lane >> 3), sub-problem (lane >> 2) & 1,
@@ -156,17 +170,32 @@ __device__ __forceinline__ void exchange16(cpair (&v)[16], uint32_t tx) {
             tmem_st2(tx + 16 * t + 8 * (q & 1) + 2 * (q >> 1), y[(t & 2) + (q >> 2)][4 * (q & 3) + 2 * (t & 1)],
                      y[(t & 2) + (q >> 2)][4 * (q & 3) + 2 * (t & 1) + 1]);
     tmem_wait_st();
+    // y[2 H + u][4 Q + 2 K + p]: point 8 u + 4 (Q >> 1) + 2 H + K, word 2 (Q & 1) + p;
+    // the first stage of pass 2 on the points of H = 0 while those of H = 1 are on their way
+    tmem_ld16x32(tx, y[0]);
+    tmem_ld16x32(tx + 32, y[1]);
+    tmem_wait_ld16(y[0]);
+    tmem_wait_ld16(y[1]);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) tmem_ld16x32(tx + ((16u * (e >> 1)) << 16) + 32 * (e & 1), y[e]);
+    for (int H = 0; H < 2; ++H) {
+        if (H == 0) {
+            tmem_ld16x32(tx + (16u << 16), y[2]);
+            tmem_ld16x32(tx + (16u << 16) + 32, y[3]);
+        } else {
+            tmem_wait_ld16(y[2]);
+            tmem_wait_ld16(y[3]);
+        }
 #pragma unroll
-    for (int e = 0; e < 4; ++e) tmem_wait_ld16(y[e]);
-    // y[2 H + u][4 Q + 2 K + p]: point 8 u + 4 (Q >> 1) + 2 H + K, word 2 (Q & 1) + p
+        for (int k1 = 2 * H; k1 < 2 * H + 2; ++k1) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const uint32_t(&z)[16] = y[(i & 2) + (i >> 3)];
-        const int o = 4 * (2 * ((i >> 2) & 1)) + 2 * (i & 1);
-        v[i].re = make_float2(__uint_as_float(z[o]), __uint_as_float(z[o + 1]));
-        v[i].im = make_float2(__uint_as_float(z[o + 4]), __uint_as_float(z[o + 5]));
+            for (int i = k1; i < 16; i += 4) {
+                const uint32_t(&z)[16] = y[(i & 2) + (i >> 3)];
+                const int o = 4 * (2 * ((i >> 2) & 1)) + 2 * (i & 1);
+                v[i].re = make_float2(__uint_as_float(z[o]), __uint_as_float(z[o + 1]));
+                v[i].im = make_float2(__uint_as_float(z[o + 4]), __uint_as_float(z[o + 5]));
+            }
+            dft4(v[k1], v[k1 + 4], v[k1 + 8], v[k1 + 12]);
+        }
     }
 }
 
@@ -514,13 +543,11 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
             tmem_ld16(tcol + 112, xb);
 #pragma unroll
             for (int q = 8; q < 12; ++q) v[order1(q)] = mul_tw(v[order1(q)], xa, q - 8);
-            send16(v, tseg + TMX, 2);
             tmem_wait_ld16(xb);
 #pragma unroll
             for (int q = 12; q < 15; ++q) v[order1(q)] = mul_tw(v[order1(q)], xb, q - 12);
-            send16(v, tseg + TMX, 3);
             exchange16(v, tseg + TMX);
-            dft16(v);
+            dft16_rest(v);
             float2 P[16];
 #pragma unroll
             for (int r = 0; r < RK; ++r) P[r] = fma2(v[r].re, v[r].re, mul2(v[r].im, v[r].im));

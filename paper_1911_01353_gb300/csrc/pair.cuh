@@ -63,11 +63,10 @@ __device__ __forceinline__ void dft8(cpair &a0, cpair &a1, cpair &a2, cpair &a3,
     a7 = axpy(kRsqrt2, s, c3);
 }
 
-// y_r = sum_k a_k exp(2 pi i k r / 16): the 4 x 4 split of dft16 in fft.cuh
-__device__ __forceinline__ void dft16(cpair (&a)[16]) {
+// y_r = sum_k a_k exp(2 pi i k r / 16): the 4 x 4 split of dft16 in fft.cuh, after its
+// first stage (dft4 of a[k1], a[k1 + 4], a[k1 + 8], a[k1 + 12] for k1 = 0 .. 3)
+__device__ __forceinline__ void dft16_rest(cpair (&a)[16]) {
     constexpr float C1 = 0.92387953251128674f, S1 = 0.38268343236508977f;
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) dft4(a[k1], a[k1 + 4], a[k1 + 8], a[k1 + 12]);
     cpair y[16];
     {
         cpair x0 = a[0], x1 = a[1], x2 = a[2], x3 = a[3];
@@ -109,6 +108,12 @@ __device__ __forceinline__ void dft16(cpair (&a)[16]) {
     }
 #pragma unroll
     for (int i = 0; i < 16; ++i) a[i] = y[i];
+}
+
+__device__ __forceinline__ void dft16(cpair (&a)[16]) {
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) dft4(a[k1], a[k1 + 4], a[k1 + 8], a[k1 + 12]);
+    dft16_rest(a);
 }
 
 }  // namespace jerk
