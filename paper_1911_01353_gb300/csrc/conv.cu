@@ -108,7 +108,7 @@ conv_kernel(ConvArgs a) {
     const SyncNamed bar_half{1 + half, NT};
 
     // (spectrum, template group) entry of this CTA
-    const int cta = (int)blockIdx.x + a.cta_base;
+    const int cta = MODE == 1 ? (int)blockIdx.x / a.plane_parts + a.cta_base : (int)blockIdx.x;
     const int g = work_entry(a, cta);
     const int item = __ldg(&a.grp[g].item);
 #define itm (a.items + item)
@@ -119,6 +119,7 @@ conv_kernel(ConvArgs a) {
         const int g1 = te;
         te = first_at_least(a.order, tb, g1, a.t0 + a.nt);
         tb = first_at_least(a.order, tb, te, a.t0);
+        plane_part(a, tb, te);
         if (tb >= te) return;                                 // (uniform over the CTA, nothing set up yet)
     }
     const int s = (cta - __ldg(&a.grp[g].cta0)) * SEGS + half;
@@ -459,7 +460,7 @@ static cudaError_t launch_one(const ConvArgs &a, int n_ctas, cudaStream_t st) {
     auto k = conv_kernel<LOG2L, MODE, STATS, ROWS>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CC::SMEM);
     if (e != cudaSuccess) return e;
-    k<<<n_ctas, CC::THREADS, CC::SMEM, st>>>(a);
+    k<<<MODE == 1 ? n_ctas * a.plane_parts : n_ctas, CC::THREADS, CC::SMEM, st>>>(a);
     return cudaGetLastError();
 }
 

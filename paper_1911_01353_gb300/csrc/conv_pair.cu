@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     const SyncNamed bar_seg{1 + seg, NT};
 
     // (spectrum, template group) entry of this CTA
-    const int cta = (int)blockIdx.x + a.cta_base;
+    const int cta = MODE == 1 ? (int)blockIdx.x / a.plane_parts + a.cta_base : (int)blockIdx.x;
     const int g = work_entry(a, cta);
     const ItemDesc *itm = a.items + __ldg(&a.grp[g].item);
     const int V = __ldg(&a.grp[g].V), bM = __ldg(&a.grp[g].bM);
@@ -240,6 +240,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
         const int g1 = te;
         te = first_at_least(a.order, tb, g1, a.t0 + a.nt);
         tb = first_at_least(a.order, tb, te, a.t0);
+        plane_part(a, tb, te);
         if (tb >= te) return;                                 // (uniform over the CTA, nothing set up yet)
     }
     const int s = (cta - __ldg(&a.grp[g].cta0)) * SEGS + seg;
@@ -672,7 +673,7 @@ cudaError_t launch_pair(const ConvArgs &a, int n_ctas, cudaStream_t st) {
     auto k = conv_pair_kernel<MODE, STATS, ROWS>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return e;
-    k<<<n_ctas, THREADS, SMEM, st>>>(a);
+    k<<<MODE == 1 ? n_ctas * a.plane_parts : n_ctas, THREADS, SMEM, st>>>(a);
     return cudaGetLastError();
 }
 

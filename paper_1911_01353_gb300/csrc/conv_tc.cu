@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
     unsigned char *opa = sm + OFF_A + grp * OPB;              // its operand A (step 1's, then step 3's)
 
     // (spectrum, template group) entry of this CTA
-    const int cta = (int)blockIdx.x + a.cta_base;
+    const int cta = MODE == 1 ? (int)blockIdx.x / a.plane_parts + a.cta_base : (int)blockIdx.x;
     const int lo = work_entry(a, cta);
     const ItemDesc *itm = a.items + __ldg(&a.grp[lo].item);
     const int V = __ldg(&a.grp[lo].V), bM = __ldg(&a.grp[lo].bM);
@@ -236,6 +236,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
         const int g1 = te;
         te = first_at_least(a.order, tb, g1, a.t0 + a.nt);
         tb = first_at_least(a.order, tb, te, a.t0);
+        plane_part(a, tb, te);
         if (tb >= te) return;                                 // (uniform over the CTA, nothing set up yet)
     }
     const int s_base = (cta - __ldg(&a.grp[lo].cta0)) * SEGS;
@@ -738,7 +739,7 @@ cudaError_t launch_tc_one(const ConvArgs &a, int n_ctas, cudaStream_t st) {
     auto k = conv_tc_kernel<PREC, MODE, STATS, ROWS>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return e;
-    k<<<n_ctas, THREADS, SMEM, st>>>(a);
+    k<<<MODE == 1 ? n_ctas * a.plane_parts : n_ctas, THREADS, SMEM, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -66,6 +66,7 @@ struct ConvArgs {
     const ConvGroup *grp;    // [n_work + 1] (item, group) entries; grp[n_work].cta0 = total CTAs
     int32_t T, n_work;
     int32_t t0, nt;          // template range written in plane mode
+    int32_t plane_length, plane_parts;   // plane mode: templates per CTA at most, and the blocks that takes
     int32_t cta_base;        // CTA of the work list that block 0 is (plane mode skips leading groups)
     // search mode
     const int32_t *slot_beg; // [T + 1] CSR into the slot entries
@@ -117,6 +118,19 @@ __device__ __forceinline__ int first_at_least(const int32_t *order, int lo, int 
         if (__ldg(order + mid) < t) lo = mid + 1; else hi = mid;
     }
     return lo;
+}
+
+// Plane mode: the templates [tb, te) of an entry in equal parts of at most
+// plane_length; plane_parts blocks in a row take one each (none past the last).
+__device__ __forceinline__ void plane_part(const ConvArgs &a, int &tb, int &te) {
+    const int n = te - tb, y = (int)blockIdx.x % a.plane_parts, parts = (n + a.plane_length - 1) / a.plane_length;
+    if (y >= parts) {
+        te = tb;
+        return;
+    }
+    const int base = n / parts, more = n - base * parts;
+    tb += y * base + min(y, more);
+    te = tb + base + (y < more ? 1 : 0);
 }
 
 // Sites of the debug build's bounds checks (the first failing one is recorded).
@@ -246,6 +260,7 @@ struct BatchLayout {
     std::vector<int32_t> n_fund;                   // [count] fundamentals of each item (stages > 1)
     int64_t total_ctas = 0;
     int n_work = 0;
+    std::vector<jerk::ConvGroup> plane;            // one spectrum, whole bank: its groups and their end (plane rows)
     std::vector<int64_t> item_cta0;                // [count + 1] conv CTAs of each item
     std::vector<int64_t> harm0;                    // [count + 1] harmonic blocks before each item
     std::vector<int32_t> harm_ny;                  // [count] parts of an item's fundamentals

@@ -13,6 +13,7 @@
 #include <cuda_fp16.h>
 
 #include "jerk_internal.h"
+#include "parts.h"
 
 using namespace jerk;
 
@@ -173,45 +174,17 @@ int tpg_for(const jerk_plan_s *pl, int nseg, int nt) {
     return (int)std::max<int64_t>(tpg, 1);
 }
 
-// Templates per CTA of a search of n bins: whole groups, or equal parts of at
-// least kMinChunk templates where those take fewer steps.  A step is one
-// template of a CTA; setting one up takes about kSetup of them, and one CTA runs
-// per SM at a time, so whole waves count (700 001 bins, 3131 templates in four
-// groups: 508 CTAs of up to 1024 templates are four waves, the last a third full,
-// 10.40 ms; in parts 9.08).  The groups themselves stay: they fix the bank's rows and,
-// in reduced precision, where the 16-bit roundings fall.  A spectrum that does
-// not fill the chip with whole groups keeps them, since in a batch others fill
-// it.  The rule sees the spectrum's length alone, so its statistics are added in
-// the same order in every batch.
-constexpr int kMinChunk = 32, kSetup = 5;
-
-// parts a group of the plan can be cut into (sizing of the launch tables and partials)
-int max_parts(const jerk_plan_s *pl) {
-    int most = 1;
-    for (const auto &g : pl->groups) most = std::max(most, g.te - g.tb);
-    return std::max(1, most / kMinChunk);
+// The rule of parts.h for this plan.  What setting a CTA up costs, in steps: FP32
+// at L = 4096 21.5 us for one template and 2.95 for each more, 8192 28.7 and 3.65;
+// 16 bits 23.6 and 1.73; 1024 and 2048 13.3 and 1.09, 17.4 and 1.42.
+PartRule part_rule(const jerk_plan_s *pl) {
+    return PartRule{pl->sms, pl->prm.precision ? 10 : pl->log2L >= 12 ? 5 : 8, pl->max_batch > 1};
 }
 
-int chunk_for(const jerk_plan_s *pl, int64_t n) {
-    const int64_t bN = (int64_t)pl->b * n;
-    const int segs = conv_segs_per_cta(pl->log2L, pl->prm.precision);
+int largest_group(const jerk_plan_s *pl) {
     int most = 1;
     for (const auto &g : pl->groups) most = std::max(most, g.te - g.tb);
-    int best = most;
-    int64_t best_cost = INT64_MAX;
-    for (int parts = 1; parts <= max_parts(pl); ++parts) {
-        const int c = (most + parts - 1) / parts;
-        int64_t ctas = 0;
-        for (const auto &g : pl->groups)
-            ctas += ((bN + g.V - 1) / g.V + segs - 1) / segs * ((g.te - g.tb + c - 1) / c);
-        if (parts == 1 && ctas < pl->sms) break;
-        const int64_t cost = (ctas + pl->sms - 1) / pl->sms * (c + kSetup);
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = c;
-        }
-    }
-    return best;
+    return most;
 }
 
 // Group templates by filter half-width: sort by (m_t, t), cut into runs of
@@ -451,7 +424,9 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
         // conv work: this spectrum's (group, segment range) entries, item-major;
         // a sub-grid keeps, per group, the templates inside it (positions into `rows`)
         int64_t nt_item = 0;
-        const int chunk = chunk_for(pl, n[i]);
+        std::vector<ConvGroup> whole;
+        std::vector<PartGroup> sizes;
+        size_t counted = 0;                   // of those, the ones whose statistics count
         // a partial search: templates outside the range that make a row of a range fundamental
         std::vector<char> extra;
         if (range) {
@@ -463,7 +438,6 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
                         if (sl[e] > 0) extra[t] = 1;
         }
         for (int part = 0; part < (range ? 2 : 1); ++part) {
-            if (part == 1) L.stat_ctas = L.total_ctas - L.item_cta0[i];
             for (const auto &g : pl->groups) {
                 ConvGroup w = g;
                 if (sub) {
@@ -482,15 +456,25 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
                 }
                 if (part == 0) nt_item += w.te - w.tb;
                 w.item = i;
-                for (int tb = w.tb, te = w.te; tb < te; tb = w.te) {
-                    w.tb = tb;
-                    w.te = te - tb > chunk ? tb + chunk : te;
-                    w.cta0 = (int32_t)L.total_ctas;
-                    h.work.push_back(w);
-                    L.total_ctas += ((bN + g.V - 1) / g.V + segs - 1) / segs;
-                }
+                whole.push_back(w);
+                sizes.push_back({((bN + g.V - 1) / g.V + segs - 1) / segs, w.te - w.tb});
+            }
+            if (part == 0) counted = whole.size();
+        }
+        // cut into equal parts: the first `more` of a group are one template longer
+        const int length = part_length(sizes, part_rule(pl));
+        for (size_t q = 0; q < whole.size(); ++q) {
+            if (range && q == counted) L.stat_ctas = L.total_ctas - L.item_cta0[i];
+            ConvGroup w = whole[q];
+            const int parts = (int)parts_of(sizes[q].count, length), more = sizes[q].count % parts;
+            for (int u = 0; u < parts; ++u, w.tb = w.te) {
+                w.te = w.tb + sizes[q].count / parts + (u < more ? 1 : 0);
+                w.cta0 = (int32_t)L.total_ctas;
+                h.work.push_back(w);
+                L.total_ctas += sizes[q].ctas;
             }
         }
+        if (range && counted == whole.size()) L.stat_ctas = L.total_ctas - L.item_cta0[i];
         L.item_cta0[i + 1] = L.total_ctas;
         L.harm_ny[i] = harm_ny_for(pl, harm_nx_for(pl, n[i]), nf);
         L.harm0[i + 1] = L.harm0[i] + harm_nx_for(pl, n[i]) * L.harm_ny[i];
@@ -544,6 +528,21 @@ jerk_status build_layout(jerk_plan_s *pl, BatchLayout &L, const std::vector<int6
     HostTables h;
     const jerk_status s = plan_tables(pl, L, n, zm, wm, h, t_lo, t_hi);
     if (s != JERK_OK) return s;
+    L.plane.clear();
+    if (n.size() == 1 && h.rows.empty()) {
+        // plane rows: whole groups, after the search's entries
+        int64_t ctas = 0;
+        const int64_t bN = (int64_t)pl->b * n[0];
+        const int segs = conv_segs_per_cta(pl->log2L, pl->prm.precision);
+        for (size_t q = 0; q <= pl->groups.size(); ++q) {
+            ConvGroup w = q < pl->groups.size() ? pl->groups[q] : ConvGroup();
+            w.item = 0;
+            w.cta0 = (int32_t)ctas;
+            L.plane.push_back(w);
+            if (q < pl->groups.size()) ctas += ((bN + w.V - 1) / w.V + segs - 1) / segs;
+        }
+        h.work.insert(h.work.end(), L.plane.begin(), L.plane.end());
+    }
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = cudaMalloc(&L.d_items, sizeof(ItemDesc) * h.items.size());
     if (e == cudaSuccess) e = cudaMalloc(&L.d_work, sizeof(ConvGroup) * h.work.size());
@@ -620,7 +619,7 @@ jerk_status transient_layout(jerk_plan_s *pl, const std::vector<int64_t> &n, con
     if (!tt.d_buf) {
         // capacity: max_batch items, each with every group, entry, fundamental and template
         const size_t mb = (size_t)pl->max_batch;
-        tt.cap_work = (int64_t)(mb * pl->groups.size() * max_parts(pl) + 1);
+        tt.cap_work = (int64_t)mb * part_entries_bound((int64_t)pl->groups.size(), pl->T, part_rule(pl)) + 1;
         tt.cap_ent = (int64_t)(mb * std::max(pl->n_entries, 1));
         tt.cap_fund = (int64_t)(mb * std::max(pl->n_fund, 1));
         tt.cap_rows = (int64_t)(mb * pl->T);
@@ -641,17 +640,16 @@ jerk_status transient_layout(jerk_plan_s *pl, const std::vector<int64_t> &n, con
     const jerk_status s = plan_tables(pl, L, n, zm, wm, h);
     if (s != JERK_OK) return s;
     if ((int64_t)h.work.size() > tt.cap_work || (int64_t)h.rows.size() > tt.cap_rows) return JERK_ENOMEM;
-    // section offsets (capacity-sized, so the device pointers never move)
-    const size_t mb = (size_t)pl->max_batch;
+    // sections packed by what they hold, so that no more is uploaded
     char *d0 = (char *)tt.d_buf;
     size_t o = 0;
-    const size_t o_items = o;  o += align256(sizeof(ItemDesc) * mb);
-    const size_t o_work = o;   o += align256(sizeof(ConvGroup) * tt.cap_work);
-    const size_t o_soff = o;   o += align256(sizeof(int64_t) * tt.cap_ent);
-    const size_t o_slen = o;   o += align256(sizeof(int64_t) * tt.cap_ent);
-    const size_t o_fund = o;   o += align256(sizeof(FundEntry) * tt.cap_fund);
-    const size_t o_counts = o; o += align256(sizeof(double) * mb * JERK_MAX_STAGES);
-    const size_t o_rows = o;   o += align256(sizeof(int32_t) * tt.cap_rows);
+    const size_t o_items = o;  o += align256(sizeof(ItemDesc) * h.items.size());
+    const size_t o_work = o;   o += align256(sizeof(ConvGroup) * h.work.size());
+    const size_t o_soff = o;   o += align256(sizeof(int64_t) * h.soff.size());
+    const size_t o_slen = o;   o += align256(sizeof(int64_t) * h.slen.size());
+    const size_t o_fund = o;   o += align256(sizeof(FundEntry) * h.fund.size());
+    const size_t o_counts = o; o += align256(sizeof(double) * h.counts.size());
+    const size_t o_rows = o;   o += align256(sizeof(int32_t) * h.rows.size());
     const size_t o_tl = o;
     L.d_items = (ItemDesc *)(d0 + o_items);
     L.d_work = (ConvGroup *)(d0 + o_work);
@@ -916,11 +914,15 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
     // (rows, CTAs and harmonic blocks grow with n; each extra spectrum adds rounding)
     pl->slot_cap = item_rows(pl, N, params->zmax, params->wmax, 0, nullptr, nullptr, nullptr, nullptr, nullptr) +
                    (int64_t)pl->max_batch * 32 * std::max(1, pl->n_fund * JERK_MAX_HARMONIC);
-    const int64_t conv_blocks = (ctas_for(pl, N) + (int64_t)pl->max_batch * (int64_t)pl->groups.size()) * max_parts(pl);
-    const int64_t harm_blocks = kMaxParts * (harm_nx_for(pl, N) + (int64_t)pl->max_batch);
     // (a partial search by template range runs each group's templates of the range
     // and, separately, the other templates its fundamentals need: up to twice the CTAs)
-    pl->stat_part_cap = 2 * 2 * conv_blocks + 2 * (int64_t)ns * harm_blocks;
+    const PartRule rule = part_rule(pl);
+    const int64_t conv_blocks =
+        std::max(part_ctas_bound(ctas_for(pl, N) + (int64_t)pl->max_batch * (int64_t)pl->groups.size(), pl->max_batch,
+                                 largest_group(pl), rule),
+                 part_ctas_bound(2 * ctas_for(pl, N), rule));
+    const int64_t harm_blocks = kMaxParts * (harm_nx_for(pl, N) + (int64_t)pl->max_batch);
+    pl->stat_part_cap = 2 * conv_blocks + 2 * (int64_t)ns * harm_blocks;
 
     // does it fit?
     size_t free_b = 0, total_b = 0;
@@ -1253,8 +1255,8 @@ jerk_status jerk_plane(jerk_plan pl, const void *d_spec, int64_t n, int32_t t0, 
     a.items = pl->cur->d_items;
     a.bank = pl->d_bank;
     a.order = pl->d_order;
-    a.grp = pl->cur->d_work;
-    a.n_work = pl->cur->n_work;
+    a.grp = pl->cur->d_work + pl->cur->n_work + 1;
+    a.n_work = (int32_t)pl->groups.size();
     a.T = pl->T;
     a.t0 = t0;
     a.nt = nt;
@@ -1268,23 +1270,29 @@ jerk_status jerk_plane(jerk_plan pl, const void *d_spec, int64_t n, int32_t t0, 
     a.tc_const = pl->d_tc;
     a.tc_cmax = pl->d_cmax;
     // only the groups that hold a template of the range (a group's positions are
-    // in ascending t, so each CTA finds its own by binary search): filtering the
-    // whole bank for 64 of 12 261 templates at 2^18 bins took 12.5 ms, this 0.15 ms
-    int64_t first = -1, last = 0, at = 0;
-    const int64_t bN = (int64_t)pl->b * n;
-    const int segs = conv_segs_per_cta(pl->log2L, pl->prm.precision), chunk = chunk_for(pl, n);
-    for (const auto &g : pl->groups) {
-        for (int tb = g.tb, te; tb < g.te; tb = te) {
-            te = g.te - tb > chunk ? tb + chunk : g.te;
-            const int64_t end = at + ((bN + g.V - 1) / g.V + segs - 1) / segs;
-            const auto k = std::lower_bound(pl->order.begin() + tb, pl->order.begin() + te, t0);
-            if (k != pl->order.begin() + te && *k < t0 + nt) {
-                if (first < 0) first = at;
-                last = end;
-            }
-            at = end;
-        }
+    // in ascending t, so each CTA finds its own by binary search), in parts as a
+    // search of these templates alone would be cut: filtering the whole bank for 64
+    // of 12 261 templates at 2^18 bins took 12.5 ms, this 0.15 ms
+    int64_t first = -1, last = 0;
+    const std::vector<ConvGroup> &work = pl->cur->plane;
+    std::vector<PartGroup> sizes;
+    int most = 0;
+    for (size_t q = 0; q + 1 < work.size(); ++q) {
+        const auto end = pl->order.begin() + work[q].te;
+        const auto k0 = std::lower_bound(pl->order.begin() + work[q].tb, end, t0);
+        if (k0 == end || *k0 >= t0 + nt) continue;
+        if (first < 0) first = work[q].cta0;
+        last = work[q + 1].cta0;
+        const int count = (int)(std::lower_bound(k0, end, t0 + nt) - k0);
+        sizes.push_back({last - work[q].cta0, count});
+        most = std::max(most, count);
     }
+    PartRule rule = part_rule(pl);
+    rule.setup *= 2;                 // and the last row's store, under no further template
+    rule.shared = false;
+    a.plane_length = most > kMinAlone ? part_length(sizes, rule) : most;
+    a.plane_parts = (int32_t)parts_of(most, a.plane_length);
+    if ((last - first) * a.plane_parts > INT32_MAX) return JERK_ENOMEM;
     a.cta_base = (int32_t)first;
     const int n_ctas = (int)(last - first);
     JCHECK(pl->prm.precision ? launch_conv_tc(pl->prm.precision, 1, false, a, n_ctas, st)
