@@ -31,10 +31,11 @@ __device__ __forceinline__ unsigned long long power_key(float2 f) {
     return (unsigned long long)__double_as_longlong(re * re + im * im);   // non-negative: integer order = value order
 }
 
-// (float)((double)f * scale), scale = sh + sl to 2^-48.  The product as a pair
-// p + e is good to 2^-46 of it; it decides the rounding unless what is left
-// after rounding lies within 2^-18 of half a unit in the last place, the result
-// is a power of two (the unit changes there) or out of the normal range.
+// (float)((double)f * scale), scale = sh + sl to 2^-48 from 2^-100 up (below, sl
+// and then sh are subnormal and keep fewer bits).  The product as a pair p + e
+// is good to 2^-46 of it; it decides the rounding unless what is left after
+// rounding lies within 2^-18 of half a unit in the last place, the result is a
+// power of two (the unit changes there) or out of the normal range.
 __device__ __forceinline__ float scaled(float f, double scale, float sh, float sl) {
     const float p = __fmul_rn(f, sh);
     const float e = __fmaf_rn(f, sl, __fmaf_rn(f, sh, -p));
@@ -43,7 +44,9 @@ __device__ __forceinline__ float scaled(float f, double scale, float sh, float s
     const unsigned bits = __float_as_uint(r);
     const float half = __uint_as_float(bits & 0x7f800000u) * 5.9604644775390625e-8f;   // 2^-24 of r's power of two
     const float a = fabsf(r);
-    if (fabsf(left - half) > half * 3.8e-6f && (bits & 0x007fffffu) != 0u && a >= 1e-28f && a <= 1e28f) return r;
+    if (fabsf(left - half) > half * 3.8e-6f && (bits & 0x007fffffu) != 0u && a >= 1e-28f && a <= 1e28f &&
+        sh >= 0x1p-100f)
+        return r;
     return (float)((double)f * scale);
 }
 
