@@ -410,7 +410,8 @@ conv_kernel(ConvArgs a) {
     if constexpr (MODE == 0) {
 #pragma unroll
         for (int r = 0; r < 16; ++r) {
-            if (((vmask >> r) & 1u) && tb < te && !failed) {
+            // (a cell that is not a number under every template has no maximum and no argmax)
+            if (((vmask >> r) & 1u) && tb < te && !failed && mx[r] >= 0.f) {
                 const unsigned long long packed =
                     ((unsigned long long)__float_as_uint(mx[r]) << 32) |
                     (unsigned long long)(0xFFFFFFFFu - (unsigned)__ldg(a.order + tb + amx[rv + NT * r]));
