@@ -404,10 +404,14 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
             unsigned long long v[2];
 #pragma unroll
             for (int l = 0; l < 2; ++l) {
-                // (a cell that is not a number under every template has no argmax: any valid position)
+                // A cell that is not a number under every template has no maximum and no
+                // argmax (any valid position is read): 0, which replaces no other group's
+                // maximum, where the bits of -1 would replace every one.
                 const int t = __ldg(a.order + min(tb + base + (int)((am[(2 * r + l) >> 2] >> (8 * ((2 * r + l) & 3))) & 255u), te - 1));
-                v[l] = ((unsigned long long)__float_as_uint(l ? mx[r].y : mx[r].x) << 32) |
-                       (unsigned long long)(0xFFFFFFFFu - (unsigned)t);
+                const float m = l ? mx[r].y : mx[r].x;
+                v[l] = m < 0.f ? 0ull
+                               : ((unsigned long long)__float_as_uint(m) << 32) |
+                                     (unsigned long long)(0xFFFFFFFFu - (unsigned)t);
             }
             const int q = c0 / 2 + 128 * r;
             pk[q ^ ((q >> 3) & 7)] = make_ulonglong2(v[0], v[1]);

@@ -466,11 +466,11 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
         unsigned long long *M1 = itm->M1 + seg0 + r;
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
-            if (i < nvalid) {
+            // (a cell that is not a number under every template has no maximum and no argmax)
+            if (i < nvalid && mx[i] >= 0.f) {
                 const int n = 64 * (32 * gcol + i);
                 const int am = sm[OFF_AMX + 32 * GT * grp + GT * i + gt];
-                // (a cell that is not a number under every template has no argmax: any valid position)
-                const int tw = __ldg(a.order + tb + min(2 * (base + am) + grp, nt - 1));
+                const int tw = __ldg(a.order + tb + 2 * (base + am) + grp);
                 const unsigned long long packed = ((unsigned long long)__float_as_uint(mx[i] * psc) << 32) |
                                                   (unsigned long long)(0xFFFFFFFFu - (unsigned)tw);
                 if (JERK_CHECK((int64_t)seg0 + n + r < bN, a.chk, kChkTcMaxProj)) atomicMax(M1 + n, packed);

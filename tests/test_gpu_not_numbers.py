@@ -1,5 +1,5 @@
-"""Bins that are not numbers, in the FP32 filter of segments of 1024, 2048 and
-8192 cells: a segment that holds such a bin has no powers, but the
+"""Bins that are not numbers, in every filter (the FP32 ones at each segment
+length, the 16-bit ones): a segment that holds such a bin has no powers, but the
 template groups' segments start at different cells, and where some template has
 a power the max-projection is the largest of them, by the template that has it;
 where none has, it is 0.  Powers are the plane rows of the same plan."""
@@ -21,7 +21,7 @@ def pkg():
     return lib_ready()
 
 
-@pytest.mark.parametrize("seg_len,precision", [(1024, 0), (2048, 0), (8192, 0)])
+@pytest.mark.parametrize("seg_len,precision", [(1024, 0), (2048, 0), (8192, 0), (4096, 0), (0, 1), (0, 2)])
 @pytest.mark.parametrize("value", [complex(np.nan, 1.0), complex(1.0, np.inf)])
 def test_maxima_are_those_of_the_numbers(pkg, seg_len, precision, value):
     n = 40000
