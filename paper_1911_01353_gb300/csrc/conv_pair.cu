@@ -56,6 +56,7 @@
 #include "pair.cuh"
 #include "rows.cuh"
 #include "tmem.cuh"
+#include "twosum.cuh"
 
 namespace jerk {
 namespace {
@@ -379,15 +380,16 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     float2 mx[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) mx[r] = make_float2(-1.0f, -1.0f);
-    float fa0 = 0.f, fa1 = 0.f;                               // FP32 statistics partials (32 templates)
+    // FP32 statistics partials, each of 16 cells x 32 templates (even and odd cells
+    // apart: one of both was off by 1.4 times as much, RMS)
+    float2 fa = make_float2(0.f, 0.f), fq = fa;
     // their FP64 sums sit in the last four of this thread's tensor-memory columns
     auto add_stats = [&] {
         double d0, d1;
         tmem_ld_f64x2(tseg + TMSTAT, d0, d1);
-        d0 += (double)fa0;
-        d1 += (double)fa1;
+        d0 += (double)take_sum(fa);
+        d1 += (double)take_sum(fq);
         tmem_st_f64x2(tseg + TMSTAT, d0, d1);
-        fa0 = fa1 = 0.f;
     };
     if constexpr (STATS) tmem_st_f64x2(tseg + TMSTAT, 0.0, 0.0);
     // Running maxima of the templates tb + base .. into the stage-1
@@ -588,21 +590,20 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
                         for (int r = 0; r < RK; ++r)
                             if (!((vmask >> r) & 1u)) P[r] = make_float2(0.f, 0.f);
                     }
-                    // four chains (two packed), then their sum
-                    float2 a2[2], q2[2];
+                    // four packed chains, then their sum
+                    float2 a2[4], q2[4];
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
+                    for (int r = 0; r < 4; ++r) {
                         a2[r] = P[r];
                         q2[r] = mul2(P[r], P[r]);
                     }
 #pragma unroll
-                    for (int r = 2; r < RK; ++r) {
-                        a2[r & 1] = add2(a2[r & 1], P[r]);
-                        q2[r & 1] = fma2(P[r], P[r], q2[r & 1]);
+                    for (int r = 4; r < RK; ++r) {
+                        a2[r & 3] = add2(a2[r & 3], P[r]);
+                        q2[r & 3] = fma2(P[r], P[r], q2[r & 3]);
                     }
-                    const float2 as = add2(a2[0], a2[1]), qs = add2(q2[0], q2[1]);
-                    fa0 += as.x + as.y;
-                    fa1 += qs.x + qs.y;
+                    fa = add2(fa, add2(add2(a2[0], a2[1]), add2(a2[2], a2[3])));
+                    fq = add2(fq, add2(add2(q2[0], q2[1]), add2(q2[2], q2[3])));
                     if ((it & 31) == 31) add_stats();
                 }
             } else {
@@ -632,8 +633,9 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     }
     double d0 = 0.0, d1 = 0.0;
     if constexpr (STATS) {
-        add_stats();
         tmem_ld_f64x2(tseg + TMSTAT, d0, d1);
+        d0 += (double)fa.x + (double)fa.y;
+        d1 += (double)fq.x + (double)fq.y;
     }
     tmem_fence_before();
     __syncthreads();

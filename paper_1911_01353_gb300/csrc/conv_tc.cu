@@ -50,6 +50,7 @@
 #include "fft.cuh"
 #include "jerk_internal.h"
 #include "tmem.cuh"
+#include "twosum.cuh"
 
 namespace jerk {
 namespace {
@@ -388,7 +389,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
         dacc[0][tid] = 0.0;
         dacc[1][tid] = 0.0;
     }
-    float c1 = 0.f, c2 = 0.f;
+    // FP32 statistics partials, each of 16 cells x 32 templates (even and odd cells apart)
+    float2 c1 = make_float2(0.f, 0.f), c2 = c1;
     // operand rows 64 s + ka, K chunks 2 blk, 2 blk + 1 (re) and 8 more (im)
     const uint32_t a1_r0 = smem_u32(opa) + (ka >> 3) * SBO + (ka & 7) * 16 + 2 * blk * LBO;
     const uint32_t a1_r1 = a1_r0 + 8 * SBO;
@@ -607,12 +609,11 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
         }
         if constexpr (MODE == 0 && STATS) {
             const float2 as = add2(a2[0], a2[1]), qs = add2(q2[0], q2[1]);
-            c1 += as.x + as.y;
-            c2 += qs.x + qs.y;
+            c1 = add2(c1, as);
+            c2 = add2(c2, qs);
             if ((i0 & 31) == 31) {
                 // unscaled: the segment's scale is applied once, at the end
-                add_f64_pair(&dacc[0][tid], &dacc[1][tid], c1, c2);
-                c1 = c2 = 0.f;
+                add_f64_pair(&dacc[0][tid], &dacc[1][tid], take_sum(c1), take_sum(c2));
             }
         }
     };
@@ -697,8 +698,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
     if constexpr (MODE == 0) {
         if (!fail && ng > 0) flush_max((ng - 1) / kFlush * kFlush);
         if constexpr (STATS) {
-            double d1 = (dacc[0][tid] + (double)c1) * (double)psc;
-            double d2 = (dacc[1][tid] + (double)c2) * ((double)psc * (double)psc);
+            double d1 = (dacc[0][tid] + ((double)c1.x + (double)c1.y)) * (double)psc;
+            double d2 = (dacc[1][tid] + ((double)c2.x + (double)c2.y)) * ((double)psc * (double)psc);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 d1 += __shfl_xor_sync(0xffffffffu, d1, o);

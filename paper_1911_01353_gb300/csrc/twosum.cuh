@@ -12,4 +12,14 @@ __device__ __forceinline__ float two_sum(float &s, float y) {
     return e;
 }
 
+// The rounded sum of a partial's two lanes; what the rounding left (of a finite
+// sum) stays as the next partial's start, so that one FP64 addition per partial
+// loses nothing.
+__device__ __forceinline__ float take_sum(float2 &v) {
+    float t = v.x;
+    const float e = two_sum(t, v.y);
+    v = make_float2(fabsf(t) <= 3.402823466e38f ? e : 0.f, 0.f);
+    return t;
+}
+
 }  // namespace jerk
