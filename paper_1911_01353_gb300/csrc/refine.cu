@@ -24,14 +24,22 @@
 // 0.05 M for the bins.  All in FP32 but the panels' phases, whose large part is
 // reduced in FP64 once per panel; the product of slope and offset inside a
 // panel (up to 10 cycles) is kept as an exact pair.  Bins are summed as exact
-// pairs.  40 candidates x 175 points (z = 200, w = 600 bank, 2^18 bins), host
-// included: 2.69 -> 0.50 ms; relative error of the powers against FP64 1.2e-7
-// before, 1.0e-7 now.
+// pairs.  Where the power sits in one or two bins nothing averages the roundings
+// of a bin: at J = 2 and 4 a bin's node pairs are summed in four chains and its
+// products' errors kept, above in two chains.  40 candidates x 175 points (z = 200,
+// w = 600 bank, 2^18 bins), host included: 2.69 -> 0.50 ms.  Relative error of a
+// strong signal's power against FP64, RMS, in 1e-7:
+//   (z, w)                            (0, 0)  (0, 20)  (4, 0)  (20, 60)  (50, 300)  (200, 600)
+//   every node summed at every bin      1.1     2.5     2.5     1.0        0.8        0.9
+//   one chain, plain products           2.1     2.4     1.4     0.9        0.9        0.7
+//   this                                0.8     1.0     0.6     0.5        0.7        0.6
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "jerk_internal.h"
+#include "twosum.cuh"
 
 namespace jerk {
 namespace {
@@ -79,12 +87,13 @@ __global__ void window_table_kernel(float2 *tab, int J, int len, const double2 *
     tab[(int64_t)i * len + k] = make_float2((float)c, (float)s);
 }
 
-// add y to the unevaluated pair (s, c): s the rounded sum, c its exact errors (Knuth's TwoSum)
-__device__ __forceinline__ void pair_add(float &s, float &c, float y) {
-    const float t = __fadd_rn(s, y);
-    const float b = __fsub_rn(t, s);
-    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(y, b)));
-    s = t;
+// add y to the unevaluated pair (s, c): s the rounded sum, c the sum of its exact errors
+__device__ __forceinline__ void pair_add(float &s, float &c, float y) { c = __fadd_rn(c, two_sum(s, y)); }
+// the same of the product x y, whose rounding error is exact too
+__device__ __forceinline__ void pair_add_product(float &s, float &c, float x, float y) {
+    const float t = __fmul_rn(x, y);
+    pair_add(s, c, t);
+    c = __fadd_rn(c, __fmaf_rn(x, y, -t));
 }
 
 __global__ void __launch_bounds__(kThreads) power_at_kernel(const float2 *__restrict__ F, int64_t N,
@@ -111,7 +120,7 @@ __global__ void __launch_bounds__(kThreads) power_at_kernel(const float2 *__rest
     float4 *panel = reinterpret_cast<float4 *>(sm + J);          // (J is even)
     float2 *chirp = sm + 3 * J;
     int ib = kPairs;
-    while (ib > 1 && 3 * J + 4 * ib * J > smem_float2) ib >>= 1;
+    while (ib > 2 && 3 * J + 4 * ib * J > smem_float2) ib >>= 1;     // (two chains below: at least two)
     float2 *S = chirp + 2 * ib * J, *D = S + ib * J;
     const float w6 = (float)(w / 6.0);
     for (int k = threadIdx.x; k < J; k += kThreads) {
@@ -184,36 +193,61 @@ __global__ void __launch_bounds__(kThreads) power_at_kernel(const float2 *__rest
         __syncthreads();
         // bins of one residue e mod J share S and D: kRun of them per thread and step
         const int runs = (nk + kRun * J - 1) / (kRun * J);
-        for (int n = threadIdx.x; n < runs * J; n += kThreads) {
-            const int b = n / J, e = n - b * J;
-            const int kap = e + b * kRun * J;
-            float rr[kRun], ri[kRun];
-            int at[kRun];
-#pragma unroll
-            for (int v = 0; v < kRun; ++v) {
-                rr[v] = ri[v] = 0.f;
-                at[v] = min(kap + v * J, nk - 1);
-            }
-            for (int p = 0; p < ib; ++p) {
-                const float2 s = S[p * J + e], d = D[p * J + e];
-                const float2 *row = tab + (int64_t)(q0 + p) * len;
+        auto bins = [&](auto chains) {                           // chains divide ib, a power of two
+            constexpr int CH = decltype(chains)::value;
+            for (int n = threadIdx.x; n < runs * J; n += kThreads) {
+                const int b = n / J, e = n - b * J;
+                const int kap = e + b * kRun * J;
+                float cr[kRun][CH], ci[kRun][CH];
+                int at[kRun];
 #pragma unroll
                 for (int v = 0; v < kRun; ++v) {
-                    const float2 cs = __ldg(row + at[v]);
-                    rr[v] = fmaf(cs.x, s.x, fmaf(cs.y, d.y, rr[v]));
-                    ri[v] = fmaf(cs.x, s.y, fmaf(-cs.y, d.x, ri[v]));
+#pragma unroll
+                    for (int u = 0; u < CH; ++u) cr[v][u] = ci[v][u] = 0.f;
+                    at[v] = min(kap + v * J, nk - 1);
+                }
+                for (int p0 = 0; p0 < ib; p0 += CH) {
+#pragma unroll
+                    for (int u = 0; u < CH; ++u) {
+                        const float2 s = S[(p0 + u) * J + e], d = D[(p0 + u) * J + e];
+                        const float2 *row = tab + (int64_t)(q0 + p0 + u) * len;
+#pragma unroll
+                        for (int v = 0; v < kRun; ++v) {
+                            const float2 cs = __ldg(row + at[v]);
+                            cr[v][u] = fmaf(cs.x, s.x, fmaf(cs.y, d.y, cr[v][u]));
+                            ci[v][u] = fmaf(cs.x, s.y, fmaf(-cs.y, d.x, ci[v][u]));
+                        }
+                    }
+                }
+#pragma unroll
+                for (int v = 0; v < kRun; ++v) {
+                    if (kap + v * J >= nk) continue;
+                    const float2 ph = __ldg(tab + (int64_t)kPairs * len + at[v]);
+                    const float2 f = F[k0 + at[v]];
+                    float rr = cr[v][0], ri = ci[v][0];
+                    if constexpr (CH == 2) rr += cr[v][1], ri += ci[v][1];
+                    if constexpr (CH == 4) {
+                        rr = (cr[v][0] + cr[v][1]) + (cr[v][2] + cr[v][3]);
+                        ri = (ci[v][0] + ci[v][1]) + (ci[v][2] + ci[v][3]);
+                    }
+                    const float xr = fmaf(rr, ph.x, -ri * ph.y), xi = fmaf(rr, ph.y, ri * ph.x);
+                    if constexpr (CH == 4) {                         // F conj(rho)
+                        pair_add_product(ar, er, f.x, xr);
+                        pair_add_product(ar, er, f.y, xi);
+                        pair_add_product(ai, ei, f.y, xr);
+                        pair_add_product(ai, ei, -f.x, xi);
+                    } else {
+                        pair_add(ar, er, fmaf(f.x, xr, f.y * xi));
+                        pair_add(ai, ei, fmaf(f.y, xr, -f.x * xi));
+                    }
                 }
             }
-#pragma unroll
-            for (int v = 0; v < kRun; ++v) {
-                if (kap + v * J >= nk) continue;
-                const float2 ph = __ldg(tab + (int64_t)kPairs * len + at[v]);
-                const float xr = fmaf(rr[v], ph.x, -ri[v] * ph.y), xi = fmaf(rr[v], ph.y, ri[v] * ph.x);
-                const float2 f = F[k0 + at[v]];
-                pair_add(ar, er, fmaf(f.x, xr, f.y * xi));       // F conj(rho)
-                pair_add(ai, ei, fmaf(f.y, xr, -f.x * xi));
-            }
-        }
+        };
+        // (classes of J = 2 and 4: the power sits in one or two bins)
+        if (J <= 4)
+            bins(std::integral_constant<int, 4>{});
+        else
+            bins(std::integral_constant<int, 2>{});
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -296,9 +330,10 @@ jerk_status power_at_host(jerk_plan pl, const float2 *F, int64_t n, const std::v
         tab += (int64_t)(kPairs + 1) * ct.len[c];
         jmax = std::max(jmax, ct.J[c]);
     }
-    // shared memory: all node pairs at once up to 96 KB (J = 64), then fewer at a time
+    // shared memory: all node pairs at once up to 96 KB (J = 64), then fewer at a time, two
+    // at least (J = 1536, the most: 132 KB)
     const int all = (3 + 4 * kPairs) * jmax, cap = (96 << 10) / (int)sizeof(float2);
-    const int smem_float2 = std::max(std::min(all, cap), 7 * jmax);
+    const int smem_float2 = std::max(std::min(all, cap), 11 * jmax);
     const size_t smem = (size_t)smem_float2 * sizeof(float2);
     // one buffer: points | tables | powers
     const size_t b_pts = (sizeof(double) * pts.size() + 255) & ~(size_t)255;
