@@ -74,9 +74,14 @@ struct ClassTables {
     int32_t J[kClasses], len[kClasses];
 };
 
-// rows i < 32: (cos, sin) of pi kappa x_i / J, x_i the positive nodes; row 32:
-// (-1)^kappa e^{-pi i kappa / J}
-__global__ void window_table_kernel(float2 *tab, int J, int len, const double2 *__restrict__ gl) {
+// The tables of every class in use (grid plane z: the z-th), one launch: a call for
+// few points is its launches.  Rows i < 32: (cos, sin) of pi kappa x_i / J, x_i the
+// positive nodes; row 32: (-1)^kappa e^{-pi i kappa / J}
+__global__ void window_table_kernel(float2 *tables, ClassTables ct, const double2 *__restrict__ gl) {
+    int cls = 0;
+    for (int z = (int)blockIdx.z; ct.J[cls] == 0 || z-- > 0;) ++cls;
+    const int J = ct.J[cls], len = ct.len[cls];
+    float2 *tab = tables + ct.off[cls];
     const int k = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
     if (k >= len) return;
     double s, c;
@@ -323,12 +328,14 @@ jerk_status power_at_host(jerk_plan pl, const float2 *F, int64_t n, const std::v
         ct.len[c] = std::max(ct.len[c], win);
     }
     int64_t tab = 0;
-    int jmax = 2;
+    int jmax = 2, classes = 0, longest = 0;
     for (int c = 0; c < kClasses; ++c) {
         if (!ct.J[c]) continue;
         ct.off[c] = tab;
         tab += (int64_t)(kPairs + 1) * ct.len[c];
         jmax = std::max(jmax, ct.J[c]);
+        longest = std::max(longest, ct.len[c]);
+        ++classes;
     }
     // shared memory: all node pairs at once up to 96 KB (J = 64), then fewer at a time, two
     // at least (J = 1536, the most: 132 KB)
@@ -344,10 +351,9 @@ jerk_status power_at_host(jerk_plan pl, const float2 *F, int64_t n, const std::v
     float2 *d_tab = (float2 *)(buf + b_pts);
     float *d_out = (float *)(buf + b_pts + b_tab);
     cudaError_t e = cudaMemcpyAsync(d_pts, pts.data(), sizeof(double) * pts.size(), cudaMemcpyHostToDevice, st);
-    for (int c = 0; c < kClasses && e == cudaSuccess; ++c) {
-        if (!ct.J[c]) continue;
-        const dim3 grid((unsigned)((ct.len[c] + 127) / 128), kPairs + 1);
-        window_table_kernel<<<grid, 128, 0, st>>>(d_tab + ct.off[c], ct.J[c], ct.len[c], pl->d_gl);
+    if (e == cudaSuccess) {
+        const dim3 grid((unsigned)((longest + 127) / 128), kPairs + 1, (unsigned)classes);
+        window_table_kernel<<<grid, 128, 0, st>>>(d_tab, ct, pl->d_gl);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
