@@ -300,7 +300,8 @@ class Plan:
         recs, stats = [], []
         cnt = float(T) * float(bN)
         size = CANDIDATE_DTYPE.itemsize
-        out = torch.empty((len(H), cap * size), dtype=torch.uint8, device=dev)
+        room = min(int(cap), bN)                         # no stage has a peak at every cell
+        out = torch.empty((len(H), room * size), dtype=torch.uint8, device=dev)
         cnt_d = torch.empty(len(H), dtype=torch.int64, device=dev)
         for si, (s1, s2) in enumerate(sums.cpu().tolist()):
             mu = s1 / cnt
@@ -308,7 +309,7 @@ class Plan:
             theta = float(np.float32(mu + float(p.thresh[si]) * sd)) if p.thresh_mode == THRESH_SIGMA \
                 else float(np.float32(p.thresh[si]))
             peaks_noalloc(maxprojs[si].data_ptr(), bN, theta, H[si], int(p.zmax), int(p.dz), int(p.wmax), int(p.dw),
-                          out[si].data_ptr(), cap, cnt_d[si:].data_ptr(), stream)
+                          out[si].data_ptr(), room, cnt_d[si:].data_ptr(), stream)
             stats.append((mu, sd, theta))
         torch.cuda.synchronize(self.device)
         for si, k in enumerate(cnt_d.cpu().tolist()):
