@@ -3,7 +3,7 @@
 // The bank's groups fix its rows and, in reduced precision, where the 16-bit
 // roundings fall; a CTA takes a whole group or one of equal parts of it.  Time
 // is counted in steps, one template of one CTA; setting a CTA up costs `setup` of
-// them, and one CTA runs per SM at a time.  The part length is the one whose
+// them, and `slots` CTAs run at a time.  The part length is the one whose
 // CTAs finish first on an idle chip, given the templates of every group that this
 // spectrum searches (a sub-grid or a template range holds the narrow groups whole
 // and few templates of the others): the longest CTA bounds a short spectrum,

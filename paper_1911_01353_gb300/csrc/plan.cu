@@ -176,9 +176,13 @@ int tpg_for(const jerk_plan_s *pl, int nseg, int nt) {
 
 // The rule of parts.h for this plan.  What setting a CTA up costs, in steps: FP32
 // at L = 4096 21.5 us for one template and 2.95 for each more, 8192 28.7 and 3.65;
-// 16 bits 23.6 and 1.73; 1024 and 2048 13.3 and 1.09, 17.4 and 1.42.
+// 16 bits 23.6 and 1.73; 1024 and 2048 13.3 and 1.09, 17.4 and 1.42.  An SM holds four
+// CTAs at L = 1024, two at 2048, one else (2048, 1581 templates, 2^18 bins: counting one
+// took 2.39 ms, two 2.25; 2^14 bins 0.31 and 0.24).
 PartRule part_rule(const jerk_plan_s *pl) {
-    return PartRule{pl->sms, pl->prm.precision ? 10 : pl->log2L >= 12 ? 5 : 8, pl->max_batch > 1};
+    const bool small = !pl->prm.precision && pl->log2L < 12;
+    return PartRule{pl->sms * (small ? 1 << (12 - pl->log2L) : 1), pl->prm.precision ? 10 : small ? 8 : 5,
+                    pl->max_batch > 1};
 }
 
 int largest_group(const jerk_plan_s *pl) {
