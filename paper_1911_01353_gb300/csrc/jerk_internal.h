@@ -333,6 +333,7 @@ struct jerk_plan_s {
     std::vector<int32_t> ent_f, ent_h, fund_t, fund_top;
     std::vector<int32_t> fh_entry;     // [n_fund][JERK_MAX_HARMONIC] -> entry (or -1)
     int32_t max_batch = 1;
+    bool batched = false;              // the bank was made by a plan for several spectra (parts.h)
     std::vector<BatchLayout *> layouts;   // tables of recently used sets of lengths (LRU)
     BatchLayout *cur = nullptr;           // tables of the last search
     BatchLayout transient_layout;         // host side of the transient tables

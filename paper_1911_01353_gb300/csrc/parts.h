@@ -13,10 +13,12 @@
 // (whole calls).
 //
 // A plan for several spectra runs them together, and there each extra CTA's setup
-// is lost time; its items are cut to parts of kMinPart templates or more, while the
-// setups add no more than 1/kSharedCost to the item's steps.  Nothing but the
-// plan's sizes and the item itself enters, so that an item's statistics are added
-// in the same order alone and in every batch.
+// is lost time: its items are cut to 32 templates or more while the setups add no
+// more than 1/24 to the item's steps, those of a plan for one spectrum to 4 (fewer
+// are setup only: one CTA takes 30.7 us for 4 templates, 21.5 for one) while they add
+// no more than half.  Nothing but the bank's plan and the item itself enters, so
+// that an item's statistics are added in the same order alone, in every batch, and
+// by every plan on the bank.
 #pragma once
 
 #include <algorithm>
@@ -25,8 +27,7 @@
 
 namespace jerk {
 
-constexpr int kMinPart = 32, kSharedCost = 24, kTried = 8;
-constexpr int kMinAlone = 4;         // a plan for one spectrum: fewer templates are setup only (4: 30.7 us, 1: 21.5)
+constexpr int kTried = 8;
 constexpr int kPartWaves = 24;       // an item is cut to at most this many waves of CTAs (or twice its whole groups)
 
 // a group's share of one item: `ctas` CTAs (of segments) walk `count` templates
@@ -38,8 +39,13 @@ struct PartGroup {
 struct PartRule {
     int slots;                       // CTAs that run at a time
     int setup;                       // steps that setting one up takes
-    bool shared;                     // the plan runs several spectra at once
+    int least;                       // templates of a part at least
+    int cost;                        // added setups are at most 1 / cost of the steps (0: any)
 };
+
+inline PartRule part_rule(int slots, int setup, bool batched) {
+    return batched ? PartRule{slots, setup, 32, 24} : PartRule{slots, setup, 4, 2};
+}
 
 inline int64_t parts_of(int count, int length) { return (count + length - 1) / length; }
 
@@ -100,8 +106,8 @@ inline int part_length(const std::vector<PartGroup> &item, const PartRule &r) {
             work += g.ctas * (g.count + r.setup * p);
         }
         if (parts > 1 && n > std::max<int64_t>((int64_t)kPartWaves * r.slots, 2 * whole)) break;
-        if (parts > 1 && length < (r.shared ? kMinPart : kMinAlone)) break;
-        if (parts > 1 && r.shared && work > steps + steps / kSharedCost) break;
+        if (parts > 1 && length < r.least) break;
+        if (parts > 1 && r.cost > 0 && work > steps + steps / r.cost) break;
         const double one = (double)(length + r.setup);
         const double waves = (double)((n + r.slots - 1) / r.slots) * one;
         const double cost = n <= r.slots ? one : std::max(one, std::min(waves, (double)work / r.slots + 0.5 * one));
@@ -130,15 +136,15 @@ inline int64_t part_ctas_bound(int64_t whole, const PartRule &r) {
 
 // ... and of `items` spectra together whose whole groups, of `most` templates or
 // fewer, are `whole` CTAs at most: each item's own bound, or what the limit on the
-// setups of a shared plan lets them come to
+// setups lets them come to
 inline int64_t part_ctas_bound(int64_t whole, int64_t items, int most, const PartRule &r) {
     const int64_t each = items * kPartWaves * r.slots + 2 * whole;
-    return r.shared ? std::min(each, whole + whole * (most + r.setup) / ((int64_t)kSharedCost * r.setup) + items) : each;
+    return r.cost > 0 ? std::min(each, whole + whole * (most + r.setup) / ((int64_t)r.cost * r.setup) + items) : each;
 }
 
 // launch-table entries of an item of `templates` templates in `groups` groups
 inline int64_t part_entries_bound(int64_t groups, int64_t templates, const PartRule &r) {
-    return r.shared ? groups + templates / kMinPart : templates;
+    return groups + templates / r.least;
 }
 
 }  // namespace jerk

@@ -179,10 +179,10 @@ int tpg_for(const jerk_plan_s *pl, int nseg, int nt) {
 // 16 bits 23.6 and 1.73; 1024 and 2048 13.3 and 1.09, 17.4 and 1.42.  An SM holds four
 // CTAs at L = 1024, two at 2048, one else (2048, 1581 templates, 2^18 bins: counting one
 // took 2.39 ms, two 2.25; 2^14 bins 0.31 and 0.24).
-PartRule part_rule(const jerk_plan_s *pl) {
+PartRule plan_rule(const jerk_plan_s *pl) {
     const bool small = !pl->prm.precision && pl->log2L < 12;
-    return PartRule{pl->sms * (small ? 1 << (12 - pl->log2L) : 1), pl->prm.precision ? 10 : small ? 8 : 5,
-                    pl->max_batch > 1};
+    return part_rule(pl->sms * (small ? 1 << (12 - pl->log2L) : 1), pl->prm.precision ? 10 : small ? 8 : 5,
+                     pl->batched);
 }
 
 int largest_group(const jerk_plan_s *pl) {
@@ -466,7 +466,7 @@ jerk_status plan_tables(jerk_plan_s *pl, BatchLayout &L, const std::vector<int64
             if (part == 0) counted = whole.size();
         }
         // cut into equal parts: the first `more` of a group are one template longer
-        const int length = part_length(sizes, part_rule(pl));
+        const int length = part_length(sizes, plan_rule(pl));
         for (size_t q = 0; q < whole.size(); ++q) {
             if (range && q == counted) L.stat_ctas = L.total_ctas - L.item_cta0[i];
             ConvGroup w = whole[q];
@@ -623,7 +623,7 @@ jerk_status transient_layout(jerk_plan_s *pl, const std::vector<int64_t> &n, con
     if (!tt.d_buf) {
         // capacity: max_batch items, each with every group, entry, fundamental and template
         const size_t mb = (size_t)pl->max_batch;
-        tt.cap_work = (int64_t)mb * part_entries_bound((int64_t)pl->groups.size(), pl->T, part_rule(pl)) + 1;
+        tt.cap_work = (int64_t)mb * part_entries_bound((int64_t)pl->groups.size(), pl->T, plan_rule(pl)) + 1;
         tt.cap_ent = (int64_t)(mb * std::max(pl->n_entries, 1));
         tt.cap_fund = (int64_t)(mb * std::max(pl->n_fund, 1));
         tt.cap_rows = (int64_t)(mb * pl->T);
@@ -920,7 +920,7 @@ jerk_status plan_memory(jerk_plan_s *pl, bool own_bank) {
                    (int64_t)pl->max_batch * 32 * std::max(1, pl->n_fund * JERK_MAX_HARMONIC);
     // (a partial search by template range runs each group's templates of the range
     // and, separately, the other templates its fundamentals need: up to twice the CTAs)
-    const PartRule rule = part_rule(pl);
+    const PartRule rule = plan_rule(pl);
     const int64_t conv_blocks =
         std::max(part_ctas_bound(ctas_for(pl, N) + (int64_t)pl->max_batch * (int64_t)pl->groups.size(), pl->max_batch,
                                  largest_group(pl), rule),
@@ -1054,6 +1054,7 @@ jerk_status jerk_plan_create(const jerk_params *params, int device, jerk_plan *o
     pl->device = device;
     pl->sms = device_sms(device);
     pl->max_batch = std::max(1, params->max_batch);
+    pl->batched = pl->max_batch > 1;
     v = plan_structure(pl);
     if (v == JERK_OK) v = plan_memory(pl, true);
     if (v != JERK_OK) {
@@ -1088,6 +1089,7 @@ jerk_status jerk_plan_share(jerk_plan parent, const jerk_params *params, jerk_pl
     pl->device = parent->device;
     pl->sms = parent->sms;
     pl->max_batch = std::max(1, params->max_batch);
+    pl->batched = parent->batched;     // the same cut of groups, so the parent's statistics bit for bit
     // the parent's structure: its groups fix the tap offset baked into every bank row
     pl->b = parent->b;
     pl->nz = parent->nz;
@@ -1291,10 +1293,11 @@ jerk_status jerk_plane(jerk_plan pl, const void *d_spec, int64_t n, int32_t t0, 
         sizes.push_back({last - work[q].cta0, count});
         most = std::max(most, count);
     }
-    PartRule rule = part_rule(pl);
+    PartRule rule = plan_rule(pl);
     rule.setup *= 2;                 // and the last row's store, under no further template
-    rule.shared = false;
-    a.plane_length = most > kMinAlone ? part_length(sizes, rule) : most;
+    rule.least = 4;
+    rule.cost = 0;
+    a.plane_length = most > rule.least ? part_length(sizes, rule) : most;
     a.plane_parts = (int32_t)parts_of(most, a.plane_length);
     if ((last - first) * a.plane_parts > INT32_MAX) return JERK_ENOMEM;
     a.cta_base = (int32_t)first;

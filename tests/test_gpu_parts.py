@@ -91,3 +91,26 @@ def test_long_groups(pkg, n, group_size, precision):
         plan.search(x)
         plan.candidates()
         check(plan, rows, np.arange(plan.info.n_templates), precision)
+
+
+@pytest.mark.parametrize("n", [5003, 40001, 90001])
+@pytest.mark.parametrize("batches", [(1, 4), (4, 1)])
+def test_plans_on_one_bank_give_the_same_bits(pkg, n, batches):
+    """Statistics too (SIGMA), whatever the plans' sizes: the bank's plan decides the cut."""
+    p = pkg.make_params(40, 2, 300, 20, stages=(1, 2), thresh=(6.0, 6.0), thresh_mode=pkg.THRESH_SIGMA, max_bins=n,
+                        group_size=300, max_batch=batches[0])
+    q = pkg.make_params(40, 2, 300, 20, stages=(1, 2), thresh=(6.0, 6.0), thresh_mode=pkg.THRESH_SIGMA,
+                        max_bins=2 * n, max_batch=batches[1])
+    x = torch.from_numpy(synth.spectrum(n, 97, [synth.Signal(n / 2.5, 20.0, 0.0, 30.0, 0.3)])).cuda()
+    with pkg.Plan(p) as parent, parent.share(q) as child:
+        got = []
+        for plan in (parent, child):
+            plan.search(x)
+            found = [(c.stage, c.p, c.t, c.power) for c in plan.candidates()]
+            got.append((found, plan.stats(0), [plan.maxproj(si)[0] for si in range(2)]))
+        assert got[0][0] == got[1][0] and got[0][1] == got[1][1] and len(got[0][0]) > 0
+        assert all(np.array_equal(a, b) for a, b in zip(got[0][2], got[1][2]))
+        if max(batches) == child.params.max_batch:
+            child.search_batch([x, x[: n // 2].contiguous()])
+            child.candidates()
+            assert child.stats(0) == got[0][1]

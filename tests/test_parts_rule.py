@@ -24,7 +24,7 @@ int main() {
     int shared, items, groups, most;
     long long templates;
     while (std::scanf("%d %d %d %lld", &shared, &items, &groups, &templates) == 4) {
-        const PartRule r{152, 5, shared != 0};
+        const PartRule r = part_rule(152, 5, shared != 0);
         std::vector<PartGroup> item(groups);
         int64_t whole = 0;
         most = 1;
