@@ -19,10 +19,10 @@
 //
 // Why three segments of four warps: the passes of one segment wait on barriers
 // over its four warps only, one warp on each of the SM's four schedulers, and
-// the other two segments fill those waits; 168 registers a thread hold 16
+// the other two segments fill those waits; 166 registers a thread hold 16
 // pairs (64), factors on their way, the running maxima (32) and their 8-bit
 // argmaxima (8) without a spill.  What bounds it is latency at these 12 warps:
-// FMA 61 %, issue 54 %, shared memory 46 % of their peaks, none of them full
+// FMA 62 %, issue 54 %, shared memory 47 % of their peaks, none of them full
 // (with both exchanges in shared memory that pipe was the bound, at 71 %).  Filter alone, ms:
 //
 //                                         12 261 templates,  3131 templates,  27 391 templates,
@@ -38,6 +38,8 @@
 //   first exchange padded, not swizzled   100.1               8.58             8.84
 //   loads and stores of the second
 //   exchange under one another             99.2               8.50             8.70
+//   statistics' lanes apart, groups cut
+//   by parts.h                             98.9               8.20             8.59
 //
 // Not faster: the factors' loads issued a whole pass earlier (103.5 ms, and 104.2
 // with the spectrum's a template earlier), so their latency is hidden already.

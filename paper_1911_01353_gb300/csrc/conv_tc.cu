@@ -27,9 +27,10 @@
 // kept them in the same phase and 42 % of the issue slots busy.  The segment
 // spectra sit in tensor memory too (64 columns per thread), which makes room in
 // registers for the 32 running maxima a thread has in this layout.  Bank of
-// 12 261 templates, 2^20 bins, FP16: filter 50.3 -> 44.7 ms, results unchanged
-// bit for bit.  The bound is still latency: shared memory (operands, template,
-// twiddles and the products' own reads) 57 %, issue 42 %, tensor pipe 25 %.
+// 12 261 templates, 2^20 bins, FP16: filter 50.3 -> 44.1 ms, powers unchanged
+// bit for bit (where two templates' powers are equal after their scale, the one
+// named may be another).  The bound is still latency: shared memory (operands,
+// template, twiddles and the products' own reads) 59 %, issue 44 %, tensor pipe 28 %.
 //
 // Scaling: each segment spectrum is divided by max|X| * max|C| over the bank,
 // so |Z| <= 1 and the FP16 operands of both steps stay in range (|U'| <= 64,
