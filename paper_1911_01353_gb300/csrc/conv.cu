@@ -108,7 +108,7 @@ conv_kernel(ConvArgs a) {
     const SyncNamed bar_half{1 + half, NT};
 
     // (spectrum, template group) entry of this CTA
-    const int cta = MODE == 1 ? (int)blockIdx.x / a.plane_parts + a.cta_base : (int)blockIdx.x;
+    const int cta = MODE == 1 ? plane_cta(a) : (int)blockIdx.x;
     const int g = work_entry(a, cta);
     const int item = __ldg(&a.grp[g].item);
 #define itm (a.items + item)

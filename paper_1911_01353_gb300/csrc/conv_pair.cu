@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_pair_kernel(ConvArgs a) {
     const SyncNamed bar_seg{1 + seg, NT};
 
     // (spectrum, template group) entry of this CTA
-    const int cta = MODE == 1 ? (int)blockIdx.x / a.plane_parts + a.cta_base : (int)blockIdx.x;
+    const int cta = MODE == 1 ? plane_cta(a) : (int)blockIdx.x;
     const int g = work_entry(a, cta);
     const ItemDesc *itm = a.items + __ldg(&a.grp[g].item);
     const int V = __ldg(&a.grp[g].V), bM = __ldg(&a.grp[g].bM);

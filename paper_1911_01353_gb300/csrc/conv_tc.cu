@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_tc_kernel(ConvArgs a) {
     unsigned char *opa = sm + OFF_A + grp * OPB;              // its operand A (step 1's, then step 3's)
 
     // (spectrum, template group) entry of this CTA
-    const int cta = MODE == 1 ? (int)blockIdx.x / a.plane_parts + a.cta_base : (int)blockIdx.x;
+    const int cta = MODE == 1 ? plane_cta(a) : (int)blockIdx.x;
     const int lo = work_entry(a, cta);
     const ItemDesc *itm = a.items + __ldg(&a.grp[lo].item);
     const int V = __ldg(&a.grp[lo].V), bM = __ldg(&a.grp[lo].bM);
