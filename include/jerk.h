@@ -385,8 +385,9 @@ jerk_status jerk_plane(jerk_plan plan, const void *d_spec, int64_t n, int32_t t0
 /* After a search: device pointer to the stage-`stage_idx` max-projection of
  * spectrum `item` (0 for jerk_search), uint64[n_cells] with
  * n_cells = floor((b n - 1)/H) + 1, each entry
- * (float bits of M_H(p)) << 32 | (0xFFFFFFFF - t).  Valid until the next
- * search on the plan. */
+ * (float bits of M_H(p)) << 32 | (0xFFFFFFFF - t), or 0 where no template's
+ * sum is a number (bins that are not).  Valid until the next search on the
+ * plan. */
 jerk_status jerk_maxproj(jerk_plan plan, int32_t item, int32_t stage_idx, const uint64_t **d_out, int64_t *n_cells);
 
 /* After a search (synchronises it): for spectrum `item`, per stage mean and
